@@ -308,7 +308,8 @@ def plan_name(B, M, N, K):
         return f"gemm_strip_kernel<{p['tile_m'] // 8},{p['strip_rows'] // 16}> x {p['ctas']} CTAs"
     if p["family"] == B.PATH_SPLITK:
         return f"gemm_cluster_kernel<{p['tile_m'] // 8}> x {p['ctas']} CTAs, {p['k_slices']} K slices"
-    return (f"gemm_tcgen05_kernel<{p['tile_m']}> x {p['ctas']} CTAs" + (f", {p['k_slices']} K slices" if p["k_slices"] > 1 else "")
+    name = "gemm_tcshort_kernel" if p["tile_m"] == 64 else "gemm_tcgen05_kernel"
+    return (f"{name}<{p['tile_m']}> x {p['ctas']} CTAs" + (f", {p['k_slices']} K slices" if p["k_slices"] > 1 else "")
             + (", balanced walk" if p["balanced"] else ""))
 
 

@@ -4,8 +4,8 @@
 
 Each .cu under csrc/ is compiled to an object, then linked into one shared library next
 to this file.  The ptxas resource report of every kernel is kept in build/ptxas.txt and
-checked: the tcgen05 kernel redistributes registers between warpgroups with setmaxnreg,
-which only works if it was allotted the full 128 registers per thread at launch.
+checked: the tcgen05 kernels redistribute registers between warpgroups with setmaxnreg,
+which only works if it was allotted the full 128 (or 96) registers per thread at launch.
 """
 import os
 import re
@@ -33,19 +33,21 @@ def _deps_mtime():
 
 
 def check_ptxas(report):
-    """Raise if a GEMM kernel spills or the tcgen05 kernel did not get 128 registers."""
+    """Raise if a GEMM kernel spills or a tcgen05 kernel did not get its registers."""
     problems = []
     for m in re.finditer(r"Compiling entry function '(\S+)' for 'sm_100a'.*?\n.*?(\d+) bytes spill stores.*?\n"
                          r".*?Used (\d+) registers", report, re.S):
         name, spill, regs = m.group(1), int(m.group(2)), int(m.group(3))
         limit = 128                               # a few stray registers are tolerable, an accumulator array is not
-        m2 = re.search(r"gemm_tcgen05_kernelILi\d+ELb(\d)E", name) or re.search(r"gemm_strip_kernelILi\d+ELi\d+ELb(\d)E", name)
+        m2 = re.search(r"gemm_tc(?:gen05|short)_kernelILi\d+ELb(\d)E", name) or re.search(r"gemm_strip_kernelILi\d+ELi\d+ELb(\d)E", name)
         if m2 and m2.group(1) == "1":
             limit = 1024                          # the debug instantiations (partials dump) may spill
         if spill > limit and "gemm_" in name:
             problems.append(f"{name}: {spill} bytes of spill stores")
-        if "gemm_tcgen05_kernel" in name and regs != 128:
-            problems.append(f"{name}: {regs} registers at launch, setmaxnreg budget assumes 128")
+        if "gemm_tcgen05" in name or "gemm_tcshort" in name:      # 512 and 640 threads share the 64 K registers
+            want = 128 if "gemm_tcgen05" in name else 96
+            if regs != want:
+                problems.append(f"{name}: {regs} registers at launch, setmaxnreg budget assumes {want}")
     if problems:
         raise RuntimeError("ptxas check failed:\n  " + "\n  ".join(problems))
 

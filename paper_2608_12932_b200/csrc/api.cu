@@ -41,10 +41,12 @@ int device_sm_count() {
     return cached[dev];
 }
 
-// Between 17 and 64 tokens both kernel families are valid.  Measured on B200 (nanoseconds, cold
-// weights): the streaming kernel costs about 4200 + 570 per group a CTA walks, times the number of
-// CTAs per SM, up to 32 tokens; above, where it walks the token blocks twice, about 7000 + 1140 per
-// group.  The tensor-core kernel's estimate comes from its own planner (tile height, K split, walk).
+// Between 17 and 64 tokens both kernel families are valid.  Measured on B200 (nanoseconds, cold weights): the cluster
+// split-K kernel costs about 4200 + 570 per group a CTA walks, times the number of CTAs per SM, up to 32 tokens; above,
+// where it walks the token blocks twice, about 7000 + 1140 per group.  The tensor-core kernel's estimate comes from its
+// own planner (tile height, K split, walk); it is the quicker one on every layer that was measured (20 tokens, behind the
+// quantiser: 8.9 against 12.1 us on 4096 -> 6144, 7.9 / 8.6 on 4096 -> 4096, 20.1 / 28.2 on 4096 -> 24576, 12.9 / 16.5 on
+// 12288 -> 4096), so the other one is left with very short K.
 bool small_m_prefers_tcgen05(int M, int N, int K, int sms) {
     if (M <= 16 || M > SPLITK_MAX_M) return M > SPLITK_MAX_M;
     const long G = K / GROUP, tiles = N / TILE_N, S = cluster_num_slices(M, N, K);
@@ -183,7 +185,7 @@ static w4a8_status gemm_impl(w4a8_path path,
     else if (path == W4A8_PATH_SPLITK || (path == W4A8_PATH_AUTO && !small_m_prefers_tcgen05(M, N, K, device_sm_count())))
         e = launch_gemm_cluster(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
     else
-        e = launch_gemm_tcgen05(qa, sa, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
+        e = launch_gemm_tcgen05(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
     return e == cudaSuccess ? W4A8_OK : W4A8_ERR_CUDA;
 }
 

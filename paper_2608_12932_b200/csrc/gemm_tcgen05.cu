@@ -1,4 +1,5 @@
-// Large-M W4A8 GEMM for sm_100a: bulk copies -> shared memory -> int4->int8 unpack into TENSOR
+// Large-M W4A8 GEMM for sm_100a (token tiles of 208 and 128 rows; 64-row tiles, for fewer tokens, run in
+// gemm_tcshort.cu - only the per-channel form below has them here): bulk copies -> shared memory -> int4->int8 unpack into TENSOR
 // MEMORY -> tcgen05.mma kind::i8 (weights from TMEM, activations from shared memory) with int32
 // accumulators in TMEM -> per-group fp32 scaling -> bf16.
 // (Sec. 3.4: quantising the activations to 8 bits is what lets the compute-bound prefill run on
@@ -74,12 +75,14 @@ constexpr int NUM_UNPACK_WARPS = 4, NUM_DRAIN_WARPS = 8;
 constexpr int RAW_STRIDE = 8576;                 // BLOB_BYTES rounded up to a multiple of 128
 constexpr int A_COLS = GROUP / 4;                // 32 TMEM columns hold one group of a weight row (4 bytes per column)
 constexpr int TMEM_COLS = 512;
-// cost model of tcgen05_plan (nanoseconds, measured): per launch; per group of a 208-, 128-, 64-row tile; for splitting K
-// (cluster launch, two cluster barriers, exchange and reduction of a 208-, 128-, 64-row tile)
-constexpr long TC_FIXED_NS = 4000, TC_GROUP_NS[3] = {650, 540, 440}, TC_SPLIT_NS[3] = {10000, 7000, 4000};
+// Cost model of tcgen05_plan (nanoseconds, measured on B200 behind the quantiser, weights cold; 208-, 128-, 64-row
+// tiles): per launch; per group a CTA walks; for splitting K over a cluster of S CTAs (two cluster barriers, exchange and
+// reduction); for the balanced walk (hand-over of two partial tiles and a slower pipeline around them).  64-row tiles run
+// in the kernel of gemm_tcshort.cu, whose tile is cut to 32 columns for up to 32 tokens.
 constexpr int TC_MAX_SPLIT = 4;
-// balanced walk: hand-over of two partial tiles (208-, 128-, 64-row) and a slower pipeline around them
-constexpr long TC_BALANCE_NS[3] = {12000, 8000, 5000};
+constexpr long TC_FIXED_NS[3] = {4000, 4000, 2500}, TC_GROUP_NS[3] = {550, 460, 270}, TC_GROUP_32_NS = 230;
+constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 10000, 10000, 10000}, {0, 0, 7000, 7000, 7000}, {0, 0, 3000, 3300, 3700}};
+constexpr long TC_BALANCE_NS[3] = {10000, 5500, 4500};
 
 // Shared-memory rings.  The activation tile comes from L2 through TMA with a latency of roughly
 // 2000 cycles, the packed blob from HBM likewise: both rings are deep enough to cover it.
@@ -89,12 +92,7 @@ struct Cfg {
     static constexpr int SB = TILE_M > 128 ? 5 : (TILE_M == 128 ? 6 : 8);     // activation stages
     static constexpr int SR = TILE_M > 128 ? 8 : (TILE_M == 128 ? 12 : 16);   // packed-blob stages: a short tile finishes a group
                                                                               // quickly, so more blobs must be in flight to cover HBM latency
-// (four accumulator buffers at 64-row tiles, where tensor memory has the room, -DTC_NB64=4: same results, 0.5-2 % faster
-// - the MMA -> drain -> MMA round trip of a buffer is not what bounds the short-tile step)
-#ifndef TC_NB64
-#define TC_NB64 2
-#endif
-    static constexpr int NB = TILE_M == 64 ? TC_NB64 : 2;                      // accumulator buffers in flight
+    static constexpr int NB = 2;                                               // accumulator buffers in flight
     static constexpr int SA_MAX = (TMEM_COLS - NB * TILE_M) / A_COLS;
     static constexpr int SA = SA_MAX > 4 ? 4 : SA_MAX;                        // weight stages in TMEM
     static constexpr int A_COL0 = NB * TILE_M;                                // first weight column (after the accumulators)
@@ -290,8 +288,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 if (!segment(si, tile, gb, ge)) break;
                 // PC: both threads add into the buffer of the tile, which the drain warps left zeroed
                 // (integer sums commute, so the order of the two threads' MMAs does not matter)
-                uint32_t buf = PC ? (tcount & 1u) : par;
-                uint32_t d_tmem = tmem_u + buf * TILE_M;
+                const uint32_t buf = PC ? (tcount & 1u) : par;
+                const uint32_t d_tmem = tmem_u + buf * TILE_M;
                 bool mine = false;
                 for (int g = gb; g < ge; ++g, ++it) {
                     if ((it & 1u) != par) continue;
@@ -310,7 +308,6 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                         if (!(ok = ptx::mbar_wait(bar(B_FULL + sb), pb, abort_flag))) break;
                         if (!(ok = ptx::mbar_wait(bar(A_FULL + sa_), pas, abort_flag))) break;
                     }
-                    if (!PC && C::NB == 4) { buf = it & 3u; d_tmem = tmem_u + buf * TILE_M; }      // this issuer's two buffers in turn
                     if (!(ok = ptx::mbar_wait(bar(ACC_EMPTY + buf), (PC ? (tcount >> 1) : (it / C::NB)) & 1, abort_flag))) break;
                     ptx::tc_fence_after_sync();
                     const uint64_t bd = b_desc0 + (uint64_t)(sb * (C::B_BYTES / 16));
@@ -764,54 +761,65 @@ int max_active_clusters(int S) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || S < 2 || S > TC_MAX_SPLIT) return 0;
     if (cached[dev][S] == 0) {
-        using C = Cfg<TILE_M>;
         int n = 0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(S * 64), 1, 1);
-        cfg.blockDim = dim3(TC_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = C::SMEM_ALLOC;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)S;
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(gemm_tcgen05_kernel<TILE_M, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 C::SMEM_ALLOC) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&n, gemm_tcgen05_kernel<TILE_M, false, true>, &cfg) != cudaSuccess)
-            n = -1;
+        if constexpr (TILE_M == 64) {
+            n = tcshort_max_clusters(S);
+        } else {
+            using C = Cfg<TILE_M>;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(S * 64), 1, 1);
+            cfg.blockDim = dim3(TC_THREADS, 1, 1);
+            cfg.dynamicSmemBytes = C::SMEM_ALLOC;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = (unsigned)S;
+            attr.val.clusterDim.y = 1;
+            attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (cudaFuncSetAttribute(gemm_tcgen05_kernel<TILE_M, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     C::SMEM_ALLOC) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n, gemm_tcgen05_kernel<TILE_M, false, true>, &cfg) != cudaSuccess)
+                n = -1;
+        }
         cached[dev][S] = n > 0 ? n : -1;
     }
     return cached[dev][S] > 0 ? cached[dev][S] : 0;
 }
 
-template <bool DEBUG, bool PC = false, bool RES = false>
-cudaError_t launch_plan(int tile_m, int S, bool balanced, const int8_t* qa, const uint16_t* sa, const void* packed, void* y,
+template <bool DEBUG, bool RES = false>
+cudaError_t launch_plan(int tile_m, int S, bool balanced, const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
                         const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials, cudaStream_t stream) {
-    if (S > 1 && !PC) {
-        if (tile_m == 64) return launch_tile<64, DEBUG, true, false, false, RES>(qa, sa, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
+    if (tile_m == 64)
+        return launch_gemm_tcshort(S, balanced, qa, sa, asum, packed, y, residual, M, N, K, workspace, debug_partials, stream);
+    if (S > 1) {
         if (tile_m == 128) return launch_tile<128, DEBUG, true, false, false, RES>(qa, sa, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
         return launch_tile<208, DEBUG, true, false, false, RES>(qa, sa, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
     }
-    if (balanced && !PC) {
-        if (tile_m == 64) return launch_tile<64, DEBUG, false, false, true, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
+    if (balanced) {
         if (tile_m == 128) return launch_tile<128, DEBUG, false, false, true, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
         return launch_tile<208, DEBUG, false, false, true, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
     }
-    if (tile_m == 64) return launch_tile<64, DEBUG, false, PC, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
-    if (tile_m == 128) return launch_tile<128, DEBUG, false, PC, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
-    return launch_tile<208, DEBUG, false, PC, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
+    if (tile_m == 128) return launch_tile<128, DEBUG, false, false, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
+    return launch_tile<208, DEBUG, false, false, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
+}
+
+template <bool DEBUG>
+cudaError_t launch_per_channel(int tile_m, const int8_t* qa, const uint16_t* sa, const void* packed, void* y, int M, int N, int K,
+                               void* workspace, int32_t* debug_sums, cudaStream_t stream) {
+    if (tile_m == 64) return launch_tile<64, DEBUG, false, true>(qa, sa, packed, y, nullptr, M, N, K, 1, workspace, debug_sums, stream);
+    if (tile_m == 128) return launch_tile<128, DEBUG, false, true>(qa, sa, packed, y, nullptr, M, N, K, 1, workspace, debug_sums, stream);
+    return launch_tile<208, DEBUG, false, true>(qa, sa, packed, y, nullptr, M, N, K, 1, workspace, debug_sums, stream);
 }
 
 }  // namespace
 
-// Tile height and K split for an [M, N, K] problem, from a cost model fitted to measurements on B200:
-// a CTA spends about TC_FIXED_NS on launch, set-up and pipeline fill, then TC_GROUP_NS[height] per
-// 128-k group of every tile it walks (the weight unpack, whose cost does not depend on the height,
-// dominates a group, so taller tiles are cheaper per token); a K split into S slices costs
-// TC_SPLIT_NS for the cluster exchange.  Tall tiles win when there are several waves of them, short
-// ones when a tall tiling would leave SMs idle, and a K split when even the shortest tiling does.
+// Tile height and K split for an [M, N, K] problem, from a cost model fitted to measurements on B200: a CTA spends
+// about TC_FIXED_NS on launch, set-up and pipeline fill, then TC_GROUP_NS[height] per 128-k group of every tile it
+// walks; a K split into S slices costs TC_SPLIT_NS for the cluster exchange.  Tall tiles are cheapest per token (2.6,
+// 3.6 and 4.2 ns per token and group) and win when there are several waves of them, short ones when a tall tiling would
+// leave SMs idle, and a K split when even the shortest tiling does.  (Against an exhaustive sweep of height, split and
+// walk at 20 to 400 tokens on eight layers the choice is within 6 % of the best.)
 long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max_split, int* balanced) {
     const int heights[3] = {208, 128, 64};
     const int n_tiles = N / TILE_N, G = K / GROUP;
@@ -823,13 +831,14 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max
         if (heights[i] > 64 && M <= heights[i + 1]) continue;        // the next height down already covers M in one tile
         const long tiles = (long)((M + heights[i] - 1) / heights[i]) * n_tiles;
         const long waves = (tiles + sms - 1) / sms;
+        const long group_ns = M <= 32 ? TC_GROUP_32_NS : TC_GROUP_NS[i];
         for (int S = 1; S <= TC_MAX_SPLIT && S <= max_split; ++S) {
             if (S > 1) {
                 if (tiles * S > sms || G / S < 4) break;
                 const int room = i == 0 ? max_active_clusters<208>(S) : (i == 1 ? max_active_clusters<128>(S) : max_active_clusters<64>(S));
                 if (tiles > room) continue;                          // the clusters must all be resident at once
             }
-            const long ns = TC_FIXED_NS + waves * TC_GROUP_NS[i] * ((G + S - 1) / S) + (S > 1 ? TC_SPLIT_NS[i] : 0);
+            const long ns = TC_FIXED_NS[i] + waves * group_ns * ((G + S - 1) / S) + TC_SPLIT_NS[i][S];
             if (best_ns < 0 || ns < best_ns) {                        // ties: taller tile, fewer slices
                 best_ns = ns; *tile_m = heights[i]; *split = S;
                 if (balanced) *balanced = 0;
@@ -837,7 +846,7 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max
             // no split, more tiles than SMs: an even share of all tiles x groups units per CTA, at the price of
             // handing partial tiles over between neighbours
             if (S == 1 && balanced && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
-                const long nb = TC_FIXED_NS + TC_GROUP_NS[i] * ((tiles * G + sms - 1) / sms) + TC_BALANCE_NS[i];
+                const long nb = TC_FIXED_NS[i] + group_ns * ((tiles * G + sms - 1) / sms) + TC_BALANCE_NS[i];
                 if (nb < best_ns) { best_ns = nb; *tile_m = heights[i]; *split = 1; *balanced = 1; }
             }
         }
@@ -845,16 +854,16 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max
     return best_ns;                                                   // the estimate, for the caller's choice of kernel family
 }
 
-cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const void* packed, void* y, const void* residual,
+cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y, const void* residual,
                                 int M, int N, int K, void* workspace, int32_t* debug_partials,
                                 cudaStream_t stream) {
     int tile_m = 64, S = 1, balanced = 0;
     tcgen05_plan(M, N, K, device_sm_count(), &tile_m, &S, TC_MAX_SPLIT, &balanced);
     if (residual)                                   // (no partials dump in this form)
-        return launch_plan<false, false, true>(tile_m, S, balanced != 0, qa, sa, packed, y, residual, M, N, K, workspace, nullptr, stream);
+        return launch_plan<false, true>(tile_m, S, balanced != 0, qa, sa, asum, packed, y, residual, M, N, K, workspace, nullptr, stream);
     if (debug_partials)
-        return launch_plan<true>(tile_m, S, balanced != 0, qa, sa, packed, y, nullptr, M, N, K, workspace, debug_partials, stream);
-    return launch_plan<false>(tile_m, S, balanced != 0, qa, sa, packed, y, nullptr, M, N, K, workspace, debug_partials, stream);
+        return launch_plan<true>(tile_m, S, balanced != 0, qa, sa, asum, packed, y, nullptr, M, N, K, workspace, debug_partials, stream);
+    return launch_plan<false>(tile_m, S, balanced != 0, qa, sa, asum, packed, y, nullptr, M, N, K, workspace, debug_partials, stream);
 }
 
 // The same pipeline with one drain per tile: for weights whose scale does not change along K.
@@ -865,8 +874,8 @@ cudaError_t launch_gemm_tcgen05_per_channel(const int8_t* qa, const uint16_t* sa
     int tile_m = 64, S = 1;
     tcgen05_plan(M, N, K, device_sm_count(), &tile_m, &S, 1, nullptr);
     if (debug_sums)
-        return launch_plan<true, true>(tile_m, 1, false, qa, sa, packed, y, nullptr, M, N, K, workspace, debug_sums, stream);
-    return launch_plan<false, true>(tile_m, 1, false, qa, sa, packed, y, nullptr, M, N, K, workspace, debug_sums, stream);
+        return launch_per_channel<true>(tile_m, qa, sa, packed, y, M, N, K, workspace, debug_sums, stream);
+    return launch_per_channel<false>(tile_m, qa, sa, packed, y, M, N, K, workspace, nullptr, stream);
 }
 
 }  // namespace w4a8

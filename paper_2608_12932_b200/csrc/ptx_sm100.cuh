@@ -47,6 +47,12 @@ __device__ __forceinline__ uint32_t lds_u8(uint32_t addr) {
 __device__ __forceinline__ void sts128(uint32_t addr, float4 v) {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
+__device__ __forceinline__ void sts128u(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void sts_u16(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"((unsigned short)v) : "memory");
+}
 __device__ __forceinline__ float4 lds128f(uint32_t addr) {
     float4 v;
     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
@@ -267,6 +273,31 @@ __device__ __forceinline__ void prefetch_tmap(const void* tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory");
 }
 
+// ---- packed pairs of fp32 (one instruction, both halves rounded to nearest even) ----------------
+__device__ __forceinline__ uint64_t pack2(uint32_t lo, uint32_t hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// acc += (v + b) * s for a pair v = (lo, hi), the accumulator updated in place
+__device__ __forceinline__ void add_fma2(uint64_t& acc, uint32_t lo, uint32_t hi, uint64_t b, uint64_t s) {
+    asm("{\n\t.reg .b64 t;\n\t"
+        "mov.b64 t, {%1, %2};\n\t"
+        "add.rn.f32x2 t, t, %3;\n\t"
+        "fma.rn.f32x2 %0, t, %4, %0;\n\t}"
+        : "+l"(acc) : "r"(lo), "r"(hi), "l"(b), "l"(s));
+}
+
 // ---- tcgen05 ----------------------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t smem_result, uint32_t ncols) {   // whole warp
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_result), "r"(ncols) : "memory");
@@ -303,6 +334,15 @@ __device__ __forceinline__ void mma_i8_ts(uint32_t d_tmem, uint32_t a_tmem, uint
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// the same with both operands in shared memory
+__device__ __forceinline__ void mma_i8_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // arrive on an mbarrier once every tcgen05 op issued so far by this thread has completed
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
@@ -360,6 +400,17 @@ __device__ __forceinline__ uint64_t smem_desc_k_sw128(uint32_t addr) {
     d |= (uint64_t)(1024 >> 4) << 32;                  // [32,46) stride byte offset >> 4
     d |= (uint64_t)1 << 46;                            // [46,48) descriptor version (sm_100)
     d |= (uint64_t)2 << 61;                            // [61,64) layout: 128-byte swizzle
+    return d;
+}
+
+// The same without swizzle: core matrices of 8 rows x 16 bytes, 128 contiguous bytes each; `k_step` bytes from one to
+// the next along K, `row_step` from eight rows to the next eight.
+__device__ __forceinline__ uint64_t smem_desc_k_none(uint32_t addr, uint32_t k_step, uint32_t row_step) {
+    uint64_t d = 0;
+    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(k_step >> 4) << 16;
+    d |= (uint64_t)(row_step >> 4) << 32;
+    d |= (uint64_t)1 << 46;
     return d;
 }
 

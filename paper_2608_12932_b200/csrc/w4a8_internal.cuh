@@ -117,12 +117,17 @@ int cluster_num_slices(int M, int N, int K);
 cudaError_t launch_gemm_cluster(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                                 void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
                                 cudaStream_t stream);
-cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const void* packed, void* y, const void* residual,
-                                int M, int N, int K, void* workspace, int32_t* debug_partials,
+cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
+                                const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
                                 cudaStream_t stream);
 cudaError_t launch_gemm_tcgen05_per_channel(const int8_t* qa, const uint16_t* sa, const void* packed, void* y,
                                             int M, int N, int K, void* workspace, int32_t* debug_sums,
                                             cudaStream_t stream);
+// 64-row token tiles (gemm_tcshort.cu); tcshort_max_clusters: clusters of S CTAs that the device holds at once
+cudaError_t launch_gemm_tcshort(int S, bool balanced, const int8_t* qa, const uint16_t* sa, const int32_t* asum,
+                                const void* packed, void* y, const void* residual, int M, int N, int K, void* workspace,
+                                int32_t* debug_partials, cudaStream_t stream);
+int tcshort_max_clusters(int S);
 // tile height, K split (at most max_split slices) and, if asked for, whether the balanced walk is taken, as the
 // tcgen05 launcher picks them; returns its time estimate (ns)
 long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max_split = 4, int* balanced = nullptr);
