@@ -108,13 +108,15 @@ def _check(code, where):
 
 
 def _stream(stream):
+    """The raw stream handle (0 = the legacy default stream)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        # the current stream of the current device, without building a Stream object (0.2 against 2 us per call)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None          # the argtypes take plain integers
 
 
 def _dev(t, dtype, name):
@@ -351,17 +353,21 @@ def w4a8_linear(x, packed_w, N, workspace, group=GROUP, out=None, scratch=None, 
     _dev(x, torch.bfloat16, "x"), _dev(packed_w, torch.uint8, "packed_w"), _dev(workspace, torch.uint8, "workspace")
     M, K = x.shape
     if out is None:
-        out = torch.empty((M, N), dtype=torch.bfloat16, device=x.device)
+        out = x.new_empty((M, N))
     else:
         _dev(out, torch.bfloat16, "out")
     if scratch is None:
-        scratch = (torch.empty((M, K), dtype=torch.int8, device=x.device),
-                   torch.empty((M,), dtype=torch.float16, device=x.device),
-                   torch.empty((M, max(K // group, 1)), dtype=torch.int32, device=x.device))
-    qa, sa, asum = scratch
-    _dev(qa, torch.int8, "qa"), _dev(sa, torch.float16, "sa"), _dev(asum, torch.int32, "asum")
-    _check(lib().w4a8_linear(_ptr(x), _ptr(packed_w), _ptr(out), M, N, K, group, _ptr(qa), _ptr(sa), _ptr(asum),
-                             _ptr(workspace), workspace.numel(), _stream(stream)), "w4a8_linear")
+        # one allocation for the three: codes, group sums, token scales, each 16-byte aligned (K is a multiple of 128)
+        scales_at = M * K + 4 * M * (K // group)
+        buf = torch.empty(scales_at + 2 * M, dtype=torch.uint8, device=x.device)
+        qa = buf.data_ptr()
+        sa, asum = qa + scales_at, qa + M * K
+    else:
+        qa, sa, asum = scratch
+        _dev(qa, torch.int8, "qa"), _dev(sa, torch.float16, "sa"), _dev(asum, torch.int32, "asum")
+        qa, sa, asum = qa.data_ptr(), sa.data_ptr(), asum.data_ptr()
+    _check(lib().w4a8_linear(x.data_ptr(), packed_w.data_ptr(), out.data_ptr(), M, N, K, group, qa, sa, asum,
+                             workspace.data_ptr(), workspace.numel(), _stream(stream)), "w4a8_linear")
     return out
 
 
