@@ -68,6 +68,21 @@ bool auto_takes_strip(int M, int N, int K) {
     return M <= 8 || N / 32 >= (device_sm_count() * 5) / 4;
 }
 
+bool takes_tcgen05(int M, int N, int K) {
+    return !auto_takes_strip(M, N, K) && small_m_prefers_tcgen05(M, N, K, device_sm_count());
+}
+
+// The device's address of a buffer in pinned host memory, if it has one and a kernel can use 16-byte accesses there.
+constexpr size_t HOST_DIRECT_MAX_BYTES = 512 * 1024;
+void* pinned_device_address(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost && aligned(a.devicePointer, 16) ? a.devicePointer : nullptr;
+}
+
 size_t slices_bytes(int M, int N, int K) {
     const int m = M < SPLITK_MAX_M ? M : SPLITK_MAX_M;
     const int S = splitk_num_slices(m, N, K);
@@ -384,11 +399,22 @@ w4a8_status w4a8_linear_host(const void* x_host_bf16, void* y_host_bf16,
         return W4A8_ERR_ALIGN;
     if (workspace_bytes < w4a8_workspace_bytes(M, N, K, group)) return W4A8_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    // Small requests in pinned memory: the quantiser reads x where it is, and the kernels that store y in plain 16-byte
+    // pieces write it where it goes.  A copy engine costs the stream two hand-overs per copy, several microseconds, to
+    // move what the kernels themselves move in one or two.
+    const void* x_at = x_dev;
+    void* y_at = y_dev;
+    if ((size_t)M * K * 2 <= HOST_DIRECT_MAX_BYTES) {
+        if (void* p = pinned_device_address(x_host_bf16)) x_at = p;
+        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K)) {
+            if (void* p = pinned_device_address(y_host_bf16)) y_at = p;
+        }
+    }
+    if (x_at == x_dev && cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return W4A8_ERR_CUDA;
-    w4a8_status s = w4a8_linear(x_dev, packed_w, y_dev, M, N, K, group, qa, sa, asum, workspace, workspace_bytes, stream);
+    w4a8_status s = w4a8_linear(x_at, packed_w, y_at, M, N, K, group, qa, sa, asum, workspace, workspace_bytes, stream);
     if (s != W4A8_OK) return s;
-    if (cudaMemcpyAsync(y_host_bf16, y_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (y_at == y_dev && cudaMemcpyAsync(y_host_bf16, y_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return W4A8_ERR_CUDA;
     return W4A8_OK;
 }
