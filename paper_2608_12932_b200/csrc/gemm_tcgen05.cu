@@ -57,7 +57,9 @@
 // activation ring is free) each drain thread pushes its partials with st.shared::cluster into the
 // ring area of the CTA that owns that share of the tile (slot = pusher's rank), a second cluster
 // barrier, and the owner sums its S slots in rank order, applies the token scale and stores bf16.
-// (Pushing 16 bytes at a time into a channel-major buffer was measured slightly slower.)
+// The shares are runs of four tokens, so that a push is 16 bytes and needs no division: word by word, each with
+// its owner found by two divisions at run time, and the sums stored 2 bytes a lane, the exchange took 10 us of a 208-row
+// tile (4096 x 4096 at 200 tokens in three slices 20.2 us, now 13.3; 12288 x 4096 in four with residual 28.3, now 22.2).
 // Every wait is bounded; on expiry the CTA records W4A8_ERR_TIMEOUT, frees TMEM and exits.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -77,12 +79,12 @@ constexpr int A_COLS = GROUP / 4;                // 32 TMEM columns hold one gro
 constexpr int TMEM_COLS = 512;
 // Cost model of tcgen05_plan (nanoseconds, measured on B200 behind the quantiser, weights cold; 208-, 128-, 64-row
 // tiles): per launch; per group a CTA walks; for splitting K over a cluster of S CTAs (two cluster barriers, exchange and
-// reduction); for the balanced walk (hand-over of two partial tiles and a slower pipeline around them).  64-row tiles run
+// reduction); for the balanced walk (hand-over of two partial tiles, and CTAs out of step: its groups in per cent of the plain walk's).  64-row tiles run
 // in the kernel of gemm_tcshort.cu, whose tile is cut to 32 columns for up to 32 tokens.
 constexpr int TC_MAX_SPLIT = 4;
-constexpr long TC_FIXED_NS[3] = {4000, 4000, 2500}, TC_GROUP_NS[3] = {550, 460, 270}, TC_GROUP_32_NS = 230;
-constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 10000, 10000, 10000}, {0, 0, 7000, 7000, 7000}, {0, 0, 3000, 3300, 3700}};
-constexpr long TC_BALANCE_NS[3] = {10000, 5500, 4500};
+constexpr long TC_FIXED_NS[3] = {3500, 3200, 2500}, TC_GROUP_NS[3] = {525, 440, 255}, TC_GROUP_32_NS = 230;
+constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 4000, 4500, 5600}, {0, 0, 2800, 2800, 3400}, {0, 0, 3000, 3300, 3700}};
+constexpr long TC_BALANCE_NS[3] = {6000, 4000, 4500}, TC_BALANCE_PERCENT[3] = {104, 104, 100};
 
 // Shared-memory rings.  The activation tile comes from L2 through TMA with a latency of roughly
 // 2000 cycles, the packed blob from HBM likewise: both rings are deep enough to cover it.
@@ -142,7 +144,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     // still run, and the roles that touch activations, token scales, the workspace or the output wait below.
     ptx::pdl_launch_dependents();
     using C = Cfg<TILE_M>;
-    static_assert(!SPLIT || C::SB * C::B_BYTES >= TILE_M * TILE_N * 4 + 64, "the split-K exchange buffer lives in the activation ring");
+    static_assert(!SPLIT || C::SB * C::B_BYTES >= (TILE_M / 4 + TC_MAX_SPLIT - 1) * TILE_N * 16, "the split-K exchange buffer lives in the activation ring");
     static_assert(!(SPLIT && PC), "the per-channel form is not split along K");
     static_assert(!BAL || (!SPLIT && !PC), "the balanced walk is for the plain persistent form");
     extern __shared__ uint8_t smem_raw[];
@@ -204,14 +206,22 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     // dealt out in equal contiguous ranges, so a CTA's first and last segment may be part of a tile; the CTA
     // that holds the later groups of such a tile reaches them first (they open its range) and hands its
     // fp32 sums over through global memory to the CTA that holds the earlier groups (they close its range).
-    const long bal_lo = BAL ? ((long)blockIdx.x * total_tiles * G) / gridDim.x : 0;
-    const long bal_hi = BAL ? ((long)(blockIdx.x + 1) * total_tiles * G) / gridDim.x : 0;
+    // (warp-uniform on purpose, and said so to the compiler by the shuffles: with the range in ordinary registers the
+    // loop counters, ring indices and MMA operands of every role left the uniform datapath: +53 ALU instructions per group
+    // and scheduler, 8 to 12 % of the walk: 4096 -> 37888 at 200 tokens, whole tiles only, 43.3 us, now 40.8; plain walk 39.6)
+    int bal_tile = 0, bal_gb = 0, bal_left = 0;
+    if (BAL) {
+        const long lo = ((long)blockIdx.x * total_tiles * G) / gridDim.x, hi = ((long)(blockIdx.x + 1) * total_tiles * G) / gridDim.x;
+        bal_tile = __shfl_sync(0xFFFFFFFFu, (int)(lo / G), 0);
+        bal_gb = __shfl_sync(0xFFFFFFFFu, (int)(lo % G), 0);
+        bal_left = __shfl_sync(0xFFFFFFFFu, (int)(hi - lo), 0) + bal_gb;      // groups to the end of the range, from the first tile's start
+    }
     auto segment = [&](int idx, int& tile, int& gb, int& ge) -> bool {
         if (BAL) {
-            tile = (int)(bal_lo / G) + idx;
-            gb = idx == 0 ? (int)(bal_lo % G) : 0;
-            const long left = bal_hi - (long)tile * G;
-            ge = left < G ? (int)left : G;
+            tile = bal_tile + idx;
+            gb = idx == 0 ? bal_gb : 0;
+            const int left = bal_left - idx * G;
+            ge = left < G ? left : G;
             return gb < ge;
         }
         tile = unit + idx * num_units;
@@ -220,7 +230,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
         return tile < total_tiles;
     };
 
-    bool exchanged = false;                     // SPLIT: this thread has passed the first cluster barrier
+    bool exchanged = false;                     // SPLIT: this thread has passed the two cluster barriers
+    constexpr int RUNS = TILE_M / 4;            // SPLIT: runs of four tokens; CTA o of the cluster reduces runs run_lo(o) .. run_lo(o + 1) - 1
+    const int runs_max = SPLIT ? (RUNS + S - 1) / S : 0;
+    auto run_lo = [&](int o) { return RUNS * o / S; };
     if (warp < 4) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
         if (warp == WARP_PRODUCER && lane == 0) {
@@ -567,14 +580,75 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 // the exchange buffers; push this thread's partials to the CTAs that own them
                 ptx::cluster_sync();
                 exchanged = true;
-                // element (token t, channel n) of the tile has index t * 128 + n; the indices are dealt out to
-                // the S CTAs in contiguous chunks
-                const int chunk = (TILE_M * TILE_N + S - 1) / S;
-                const uint32_t red = smem_base + C::B_OFF;
+                // The tile's runs of four tokens are dealt out to the S CTAs; a thread pushes 16 bytes (its channel, four
+                // tokens) at a time: slot [pusher][run of the owner][channel], channels 4 apart side by side, so that the lane
+                // that sums channels 4 l .. 4 l + 3 reads beside its neighbours.
+                const int slot_n = (n_local & 3) * 32 + (n_local >> 2);
+                const int lo1 = run_lo(1), lo2 = S > 2 ? run_lo(2) : RUNS, lo3 = S > 3 ? run_lo(3) : RUNS;
 #pragma unroll
-                for (int i = 0; i < C::W; ++i) {
-                    const int idx = (h * C::W + i) * TILE_N + n_local, owner = idx / chunk;
-                    ptx::st_dsmem_f32(ptx::map_to_cta(red + (uint32_t)(slice * chunk + idx - owner * chunk) * 4u, (uint32_t)owner), facc[i]);
+                for (int i = 0; i < C::W; i += 4) {
+                    if (m_base + i < M) {
+                        const int run = h * (C::W / 4) + i / 4;
+                        const int owner = (run >= lo1) + (run >= lo2) + (run >= lo3);
+                        const int first = run >= lo3 ? lo3 : (run >= lo2 ? lo2 : (run >= lo1 ? lo1 : 0));
+                        const uint32_t at = smem_base + C::B_OFF + (uint32_t)((slice * runs_max + run - first) * TILE_N + slot_n) * 16u;
+                        ptx::st_dsmem_f32x4(ptx::map_to_cta(at, (uint32_t)owner), make_float4(facc[i], facc[i + 1], facc[i + 2], facc[i + 3]));
+                    }
+                }
+                // This CTA's share, by the drain warps: a warp takes a run at a time (four tokens x the tile's 128 channels, four
+                // to a lane, stores of 256 bytes a row; stores of 2 bytes a lane cost 8 cycles each).  The residual is asked for
+                // before the second barrier, so that its round trip runs under the exchange.
+                constexpr int ITEMS = (RUNS / 2 + NUM_DRAIN_WARPS - 1) / NUM_DRAIN_WARPS;                // S >= 2
+                const int w8 = warp - WARP_DRAIN0, lo = run_lo(slice), cnt = run_lo(slice + 1) - lo;
+                const int m_first = mtile * TILE_M + 4 * (lo + w8);                                     // items are eight runs apart
+                const size_t at0 = (size_t)m_first * N + (size_t)ntile * TILE_N + 4 * lane;
+                uint2 rr[RES ? ITEMS : 1][4];
+                if (RES) {
+#pragma unroll
+                    for (int j = 0; j < ITEMS; ++j)
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            rr[j][t] = make_uint2(0u, 0u);
+                            if (w8 + 8 * j < cnt && m_first + 32 * j + t < M)
+                                rr[j][t] = __ldcg(reinterpret_cast<const uint2*>(residual + at0 + (size_t)(32 * j + t) * N));
+                        }
+                }
+                ptx::cluster_sync();                       // release after the pushes, acquire before the sums
+                if (*abort_flag) break;
+#pragma unroll
+                for (int j = 0; j < ITEMS; ++j) {
+                    if (w8 + 8 * j < cnt && m_first + 32 * j < M) {
+                        float4 acc[4];                                                  // channel 4 lane + c: four tokens
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) acc[c] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        for (int s2 = 0; s2 < S; ++s2) {                                // rank order: deterministic
+                            const uint32_t src = smem_base + C::B_OFF + (uint32_t)((s2 * runs_max + w8 + 8 * j) * TILE_N + lane) * 16u;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const float4 v = ptx::lds128f(src + c * 512);
+                                acc[c].x += v.x; acc[c].y += v.y; acc[c].z += v.z; acc[c].w += v.w;
+                            }
+                        }
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const int m = m_first + 32 * j + t;
+                            if (m < M) {
+                                const float ts = __half2float(__ushort_as_half(__ldg(sa + m)));
+                                float f[4];
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) f[c] = t == 0 ? acc[c].x : (t == 1 ? acc[c].y : (t == 2 ? acc[c].z : acc[c].w));
+                                uint2 o;
+                                if (RES) {
+                                    o.x = ptx::pack_bf16x2(fmaf(f[0], ts, __uint_as_float(rr[j][t].x << 16)), fmaf(f[1], ts, __uint_as_float(rr[j][t].x & 0xFFFF0000u)));
+                                    o.y = ptx::pack_bf16x2(fmaf(f[2], ts, __uint_as_float(rr[j][t].y << 16)), fmaf(f[3], ts, __uint_as_float(rr[j][t].y & 0xFFFF0000u)));
+                                } else {
+                                    o.x = ptx::pack_bf16x2(f[0] * ts, f[1] * ts);
+                                    o.y = ptx::pack_bf16x2(f[2] * ts, f[3] * ts);
+                                }
+                                *reinterpret_cast<uint2*>(y + at0 + (size_t)(32 * j + t) * N) = o;
+                            }
+                        }
+                    }
                 }
                 break;                          // one tile per cluster
             }
@@ -668,30 +742,9 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     }
 
     ptx::pdl_wait();                            // every thread, before the split-K tail's stores and the status word
-    if (SPLIT) {
-        // first barrier for every thread that has not passed it in the drain role, then the second one
-        // (release after the pushes, acquire before the sums); this CTA then reduces its share of the tile
-        if (!exchanged) ptx::cluster_sync();
+    if (SPLIT && !exchanged) {                  // both barriers for every thread that has not passed them in the drain role
         ptx::cluster_sync();
-        if (unit < total_tiles && !*abort_flag) {
-            int ntile, mtile;
-            tile_of(unit, ntile, mtile);
-            const int chunk = (TILE_M * TILE_N + S - 1) / S;
-            const int lo = slice * chunk;
-            const int cnt = (TILE_M * TILE_N - lo) < chunk ? (TILE_M * TILE_N - lo) : chunk;
-            const float* red = reinterpret_cast<const float*>(smem + C::B_OFF);
-            for (int i = tid; i < cnt; i += TC_THREADS) {
-                float acc = 0.0f;
-                for (int s2 = 0; s2 < S; ++s2) acc += red[s2 * chunk + i];        // rank order: deterministic
-                const int idx = lo + i, m = mtile * TILE_M + idx / TILE_N, nn = idx % TILE_N;
-                if (m < M) {
-                    const float t = __half2float(__ushort_as_half(__ldg(sa + m)));
-                    float v = acc * t;
-                    if (RES) v += __bfloat162float(residual[(size_t)m * N + (size_t)ntile * TILE_N + nn]);
-                    y[(size_t)m * N + (size_t)ntile * TILE_N + nn] = __float2bfloat16_rn(v);
-                }
-            }
-        }
+        ptx::cluster_sync();
     }
     if (*abort_flag && lane == 0) atomicExch(status, (uint32_t)W4A8_ERR_TIMEOUT);
     ptx::tc_fence_before_sync();
@@ -846,7 +899,7 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max
             // no split, more tiles than SMs: an even share of all tiles x groups units per CTA, at the price of
             // handing partial tiles over between neighbours
             if (S == 1 && balanced && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
-                const long nb = TC_FIXED_NS[i] + group_ns * ((tiles * G + sms - 1) / sms) + TC_BALANCE_NS[i];
+                const long nb = TC_FIXED_NS[i] + group_ns * ((tiles * G + sms - 1) / sms) * TC_BALANCE_PERCENT[i] / 100 + TC_BALANCE_NS[i];
                 if (nb < best_ns) { best_ns = nb; *tile_m = heights[i]; *split = 1; *balanced = 1; }
             }
         }

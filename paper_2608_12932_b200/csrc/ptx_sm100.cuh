@@ -184,6 +184,13 @@ __device__ __forceinline__ bool wait_flag_acquire_gpu(const uint32_t* p, uint32_
     }
 }
 
+// two floats rounded to bf16, the first in the low half
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
 // ---- thread-block clusters, distributed shared memory, programmatic dependent launch -----------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;
