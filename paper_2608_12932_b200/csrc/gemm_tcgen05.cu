@@ -83,7 +83,7 @@ constexpr int TMEM_COLS = 512;
 // in the kernel of gemm_tcshort.cu, whose tile is cut to 32 columns for up to 32 tokens.
 constexpr int TC_MAX_SPLIT = 4;
 constexpr long TC_FIXED_NS[3] = {3500, 3200, 2500}, TC_GROUP_NS[3] = {525, 440, 255}, TC_GROUP_32_NS = 230;
-constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 4000, 4500, 5600}, {0, 0, 2800, 2800, 3400}, {0, 0, 3000, 3300, 3700}};
+constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 4000, 4500, 5600}, {0, 0, 2800, 2800, 3400}, {0, 0, 1800, 2700, 3500}};
 constexpr long TC_BALANCE_NS[3] = {6000, 4000, 4500}, TC_BALANCE_PERCENT[3] = {104, 104, 100};
 
 // Shared-memory rings.  The activation tile comes from L2 through TMA with a latency of roughly

@@ -23,7 +23,9 @@
 //    global memory inside the loop;
 //  * the MMA's N is the tile's own token count rounded up to 16, a drain warp whose columns lie past the last token
 //    only passes the barriers on, and up to 32 tokens the tile is cut to 32 columns;
-//  * a K split exchanges its partials 16 bytes at a time (four tokens of a channel, lanes side by side).
+//  * a K split exchanges its partials 16 bytes at a time (four tokens of a channel) and stores its sums 128 bytes a row,
+//    with the residual requested ahead of the exchange's second barrier (2 bytes a lane and the residual after it:
+//    12288 -> 4096 with residual at 64 tokens in four slices 13.4 us, now 12.7; 4096 -> 4096 in two 9.6, now 8.6).
 // Measured on B200 (one 128-channel tile per SM, slope over K): 349 -> 253 ns a group at 64 tokens, 349 -> 226 at 32
 // tokens (4.4 TB/s of weights); 64 tokens, 4096 -> 6144 behind the quantiser 14.7 -> 12.0 us, 12288 -> 4096 18.9 -> 16.1.
 // Of the parts, two groups a step alone made it slower (448 ns): it is the instruction count that has to fall.
@@ -176,7 +178,7 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
         return tile < total_tiles;
     };
 
-    bool exchanged = false;                     // SPLIT: this thread has passed the first cluster barrier
+    bool exchanged = false;                     // SPLIT: this thread has passed the two cluster barriers
     constexpr int RUNS = TILE_M / 4;            // SPLIT: runs of four tokens; CTA o of the cluster reduces runs run_lo(o) .. run_lo(o + 1) - 1
     const int runs_max = SPLIT ? (RUNS + S - 1) / S : 0;
     auto run_lo = [&](int o) { return o * RUNS / S; };
@@ -526,7 +528,9 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 ptx::cluster_sync();
                 exchanged = true;
                 // The tile's runs of four tokens are dealt out to the S CTAs; a thread pushes 16 bytes (its channel, four
-                // tokens) at a time, lanes side by side: slot [pusher][run of the owner][channel].
+                // tokens) at a time: slot [pusher][run of the owner][channel], even channels first, so that the lane that sums
+                // channels 2 p and 2 p + 1 reads beside its neighbours.
+                const int slot_n = (n_local & 1) * 64 + (n_local >> 1);
                 const int lo1 = run_lo(1), lo2 = S > 2 ? run_lo(2) : RUNS, lo3 = S > 3 ? run_lo(3) : RUNS;
 #pragma unroll
                 for (int i = 0; i < C::W; i += 4) {
@@ -534,9 +538,50 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                         const int run = (h * C::W + i) / 4;
                         const int owner = (run >= lo1) + (run >= lo2) + (run >= lo3);
                         const int first = run >= lo3 ? lo3 : (run >= lo2 ? lo2 : (run >= lo1 ? lo1 : 0));
-                        const uint32_t at = smem_base + (uint32_t)((slice * runs_max + run - first) * TILE_N + n_local) * 16u;
+                        const uint32_t at = smem_base + (uint32_t)((slice * runs_max + run - first) * TILE_N + slot_n) * 16u;
                         const float2 p0 = ptx::unpack2(facc[i / 2]), p1 = ptx::unpack2(facc[i / 2 + 1]);
                         ptx::st_dsmem_f32x4(ptx::map_to_cta(at, (uint32_t)owner), make_float4(p0.x, p0.y, p1.x, p1.y));
+                    }
+                }
+                // This CTA's share, by the drain warps: half a run at a time (four tokens x 64 channels, two to a lane, stores of
+                // 128 bytes a row).  The residual is asked for before the second barrier: its round trip runs under the exchange.
+                constexpr int ITEMS = (RUNS + NUM_DRAIN_WARPS - 1) / NUM_DRAIN_WARPS;          // S >= 2: at most RUNS / 2 runs
+                const int w8 = warp - WARP_DRAIN0, lo = run_lo(slice), cnt = 2 * (run_lo(slice + 1) - lo);
+                const int pair = (w8 & 1) * 32 + lane, m_first = mtile * TILE_M + 4 * (lo + (w8 >> 1));      // items are four runs apart
+                const size_t at0 = (size_t)m_first * N + (size_t)ntile * TILE_N + 2 * pair;
+                uint32_t rr[RES ? ITEMS : 1][4];
+                if (RES) {
+#pragma unroll
+                    for (int j = 0; j < ITEMS; ++j)
+#pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            rr[j][t] = w8 + 8 * j < cnt && m_first + 16 * j + t < M
+                                           ? __ldcg(reinterpret_cast<const uint32_t*>(residual + at0 + (size_t)(16 * j + t) * N)) : 0u;
+                }
+                ptx::cluster_sync();                       // release after the pushes, acquire before the sums
+                if (*abort_flag) break;
+#pragma unroll
+                for (int j = 0; j < ITEMS; ++j) {
+                    if (w8 + 8 * j < cnt && m_first + 16 * j < M) {
+                        float4 a0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), a1 = a0;
+                        for (int s2 = 0; s2 < S; ++s2) {                                // rank order: deterministic
+                            const uint32_t src = smem_base + (uint32_t)((s2 * runs_max + (w8 >> 1) + 4 * j) * TILE_N + pair) * 16u;
+                            const float4 v0 = ptx::lds128f(src), v1 = ptx::lds128f(src + 1024);
+                            a0.x += v0.x; a0.y += v0.y; a0.z += v0.z; a0.w += v0.w;
+                            a1.x += v1.x; a1.y += v1.y; a1.z += v1.z; a1.w += v1.w;
+                        }
+                        const float f0[4] = {a0.x, a0.y, a0.z, a0.w}, f1[4] = {a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const int m = m_first + 16 * j + t;
+                            if (m < M) {
+                                const float ts = __half2float(__ushort_as_half(__ldg(sa + m))) * SCALE_OUT;
+                                const uint32_t o = RES ? ptx::pack_bf16x2(fmaf(f0[t], ts, __uint_as_float(rr[j][t] << 16)),
+                                                                          fmaf(f1[t], ts, __uint_as_float(rr[j][t] & 0xFFFF0000u)))
+                                                       : ptx::pack_bf16x2(f0[t] * ts, f1[t] * ts);
+                                *reinterpret_cast<uint32_t*>(y + at0 + (size_t)(16 * j + t) * N) = o;
+                            }
+                        }
                     }
                 }
                 break;                          // one tile per cluster
@@ -616,34 +661,9 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     }
 
     ptx::pdl_wait();                            // every thread, before the split-K tail's stores and the status word
-    if (SPLIT) {
-        // first barrier for every thread that has not passed it in the drain role, then the second one
-        // (release after the pushes, acquire before the sums); this CTA then reduces its share of the tile
-        if (!exchanged) ptx::cluster_sync();
+    if (SPLIT && !exchanged) {                  // both barriers for every thread that has not passed them in the drain role
         ptx::cluster_sync();
-        if (unit < total_tiles && !*abort_flag) {
-            int ntile, mtile;
-            tile_of(unit, ntile, mtile);
-            const int lo = run_lo(slice), cnt = (run_lo(slice + 1) - lo) * TILE_N;
-            for (int i = tid; i < cnt; i += TS_THREADS) {
-                const int m0 = mtile * TILE_M + 4 * (lo + i / TILE_N);
-                if (m0 >= M) break;
-                float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                for (int s2 = 0; s2 < S; ++s2) {                                  // rank order: deterministic
-                    const float4 v = ptx::lds128f(smem_base + (uint32_t)(s2 * runs_max * TILE_N + i) * 16u);
-                    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-                }
-                const float f[4] = {acc.x, acc.y, acc.z, acc.w};
-                const size_t at = (size_t)m0 * N + (size_t)ntile * TILE_N + i % TILE_N;
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    if (m0 + t < M) {
-                        const float ts = __half2float(__ushort_as_half(__ldg(sa + m0 + t))) * SCALE_OUT;
-                        y[at + (size_t)t * N] = __float2bfloat16_rn(RES ? fmaf(f[t], ts, __bfloat162float(residual[at + (size_t)t * N])) : f[t] * ts);
-                    }
-                }
-            }
-        }
+        ptx::cluster_sync();
     }
     if (*abort_flag && lane == 0) atomicExch(status, (uint32_t)W4A8_ERR_TIMEOUT);
     ptx::tc_fence_before_sync();

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("K,N,tile,slices,Ms", [(13056, 8192, 128, 2, (66, 128)), (5248, 5120, 128, 3, (66, 101, 127)),
-                                                (12288, 4096, 128, 4, (65, 98, 128)), (4224, 6144, 208, 2, (193, 207)),
+                                                (17408, 4096, 128, 4, (65, 98, 128)), (4224, 6144, 208, 2, (193, 207)),
                                                 (3200, 5120, 208, 3, (193, 206)), (8448, 4096, 208, 4, (131, 193, 208))])
 def test_exchange(K, N, tile, slices, Ms):
     M_max = max(Ms)
