@@ -60,12 +60,13 @@ bool small_m_prefers_tcgen05(int M, int N, int K, int sms) {
 
 namespace {
 
-// Where w4a8_gemm takes the strip kernel: up to 8 tokens always; from 9 to 16 tokens (two token blocks per warp:
-// the activation tiles then crowd the ring of a narrow strip) only on layers wide enough for strips of 32 rows,
-// where it is measured faster than the cluster split-K kernel on B200.
+// Where w4a8_gemm takes the strip kernel: up to 8 tokens always; from 9 to 16 tokens (two token blocks per warp) unless a
+// long K meets so few strips that splitting K over a cluster pays.  Measured on B200 at 16 tokens, strip against cluster
+// kernel: 2048 -> 2048 3.1 and 6.7 us, 4096 -> 4096 5.0 and 5.6, 12288 -> 4096 9.6 and 9.8, 13824 -> 5120 12.5 and 17.7,
+// 2048 -> 1024 3.1 and 3.4; but 8192 -> 1024 5.9 and 5.0, 16384 -> 128 9.6 and 6.5.
 bool auto_takes_strip(int M, int N, int K) {
     if (!strip_supported(M, N, K)) return false;
-    return M <= 8 || N / 32 >= (device_sm_count() * 5) / 4;
+    return M <= 8 || N >= 2048 || K <= 2048;
 }
 
 bool takes_tcgen05(int M, int N, int K) {

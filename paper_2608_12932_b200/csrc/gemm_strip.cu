@@ -37,7 +37,7 @@
 //  * Launched with programmatic stream serialisation: the weight copies of the first ring fill
 //    are requested before griddepcontrol.wait, so this kernel's weight stream starts under the
 //    tail of its predecessor; activations, token scales, group sums and the workspace are touched
-//    only after the wait.  A CTA stays under half an SM's shared memory and registers, so that
+//    only after the wait.  Up to 8 tokens a CTA stays under half an SM's shared memory and registers, so that
 //    two consecutive launches are resident together.
 //  * Every wait is bounded; on expiry the CTA sets its abort flag, every role leaves its loop, the
 //    status word becomes W4A8_ERR_TIMEOUT and the kernel returns.
@@ -73,13 +73,14 @@ constexpr int ST_EPILOGUE_WARP = ST_CONSUMER_WARPS + ST_PRODUCER_WARPS;
 constexpr int ST_THREADS = (ST_CONSUMER_WARPS + ST_PRODUCER_WARPS + 1) * 32;
 constexpr int ST_MAX_STAGES = 8;
 constexpr int ST_W_BYTES = ST_CW == 8 ? 17408 : (ST_CW == 12 ? 26624 : 34816);                         // weight part of a stage (16 KB of nibbles + scales + zero points, padded)
-// CTAs per SM.  One CTA per SM with sixteen consumer warps (-DST_CW=16 -DST_MINB=1: 96 registers, no spills with two
-// token blocks, a 220 KB ring) was measured equal to 17 % slower at up to 8 tokens and equal to 10 % faster at 16
-// (the 4096 -> 24576 layer: 17.3 against 19.2 us); not worth a second build of the kernel.
-#ifndef ST_MINB
-#define ST_MINB 2
-#endif
-constexpr int ST_SMEM_BUDGET = (ST_MINB == 2 ? 112 : 220) * 1024;   // per CTA: two CTAs share an SM
+// CTAs per SM.  Up to 8 tokens two: the second CTA's warps multiply while the first one's wait for data.  With two token
+// blocks one, with twice the ring and up to 168 registers a thread: at 80 the second block's fragments and sums leave no
+// room for the loads of the next unit, and every stage waits for its shared-memory round trips in turn (4096 -> 24576 at 16
+// tokens 19.2 us with two, 17.1 with one; 5120 -> 27648 26.3 and 23.4; 12288 -> 4096 with residual 16.9 and 9.6; the other
+// way round up to 8 tokens: 4096 -> 24576 12.9 and 14.7).  Twelve or sixteen consumer warps in one CTA per SM are 2 to 20 %
+// slower on most layers.
+__host__ __device__ constexpr int st_ctas_per_sm(int mb) { return mb == 1 ? 2 : 1; }
+__host__ __device__ constexpr int st_smem_budget(int mb) { return (mb == 1 ? 112 : 220) * 1024; }
 constexpr uint32_t ST_STAY = 128;                         // one-kernel fused form: CTAs that stay to requantise (swept 32..296 on B200)
 constexpr int ST_MAX_ASUM_WORDS = 4096;                   // group sums of all tokens kept in shared memory
 
@@ -208,7 +209,7 @@ struct StripArgs {
 // FUSE == 3 is unrelated to gate+up: the plain projection with a residual added at the store (fp32 staging, the
 // residual's 16-byte pieces requested before the wait for the consumers), for the O and down projections.
 template <int MB, int RBLK, bool DEBUG, int FUSE>
-__global__ void __launch_bounds__(ST_THREADS, ST_MINB)
+__global__ void __launch_bounds__(ST_THREADS, st_ctas_per_sm(MB))
 gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_nib,
                   const __grid_constant__ CUtensorMap tm_scale, const __grid_constant__ CUtensorMap tm_zero,
                   const StripArgs a) {
@@ -805,7 +806,7 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     const int G = K / GROUP;
     const bool fp32_stage = FUSE == 3;
     const int fixed = st_layout(MB, RBLK, 0, G, fp32_stage).total + 1024;
-    int stages = (ST_SMEM_BUDGET - fixed) / st_stage_bytes(MB, RBLK);
+    int stages = (st_smem_budget(MB) - fixed) / st_stage_bytes(MB, RBLK);
     if (stages > ST_MAX_STAGES) stages = ST_MAX_STAGES;
     if (stages < 2) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)st_layout(MB, RBLK, stages, G, fp32_stage).total + 1024;
@@ -816,10 +817,10 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     static bool attr_done[64] = {false};
     static int resident[64] = {0};                          // CTAs of this instance that fit on the device at once
     if (!attr_done[dev]) {
-        e = cudaFuncSetAttribute(gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM_BUDGET);
+        e = cudaFuncSetAttribute(gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, st_smem_budget(MB));
         if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, ST_THREADS, ST_SMEM_BUDGET);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, ST_THREADS, st_smem_budget(MB));
         if (e != cudaSuccess) return e;
         resident[dev] = per_sm * device_sm_count();
         attr_done[dev] = true;
@@ -917,7 +918,7 @@ bool strip_supported(int M, int N, int K) {
 
 // Strip width and CTA count for a problem (measured on B200, sweep of widths 16..128 and 148..296 CTAs on the
 // four layer shapes of an 8B-class decoder, 4 to 16 tokens): the widest strip that still gives about 1.25 strips
-// per SM (one step narrower if a wide strip would leave SMs with a single CTA), and up to two CTAs per SM - the second CTA's warps multiply while the first one's wait for data, which is
+// per SM (one step narrower if a wide strip would leave SMs with a single CTA), and up to two CTAs per SM up to 8 tokens - the second CTA's warps multiply while the first one's wait for data, which is
 // worth more than a whole SM's shared memory held free for the next launch; the next launch's CTAs still start
 // (and prefetch) as soon as the first CTAs of this one leave.  Wide strips share an activation tile between more
 // rows (less traffic from L2 into shared memory); 16-row strips are left to up to 8 tokens, where their 16
@@ -939,7 +940,7 @@ void strip_plan(int M, int N, int K, int* strip_rows, int* ctas) {
         if (v == 16 || v == 32 || v == 64 || v == 128) R = v;
     }
 #endif
-    int limit = ST_MINB * sms;
+    int limit = st_ctas_per_sm(M <= 8 ? 1 : 2) * sms;
 #ifdef W4A8_TUNING
     if (const char* e = getenv("W4A8_STRIP_CTAS")) { const int v = atoi(e); if (v >= 1) limit = v; }
 #endif
