@@ -457,6 +457,21 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             float facc[C::W];
 #pragma unroll
             for (int i = 0; i < C::W; ++i) facc[i] = 0.0f;
+            if (BAL && ge < G) {
+                // Balanced walk: this CTA's last tile, whose later groups the next CTA summed first (they open its range): the sums
+                // start from those.  Fetched here and not after the last group they are off the tail that the launch ends with,
+                // and warp by warp (a flag bit each) they need no barrier of the CTA.  (4096 -> 24576 at 200 tokens 32.5 us, now
+                // 31.8; 12288 -> 4096 at 1024 with residual 70.5, now 69.1)
+                if (lane == 0 && !ptx::wait_bit_acquire_gpu(handover_flags + blockIdx.x + 1, 1u << (warp - WARP_DRAIN0), abort_flag)) ok = false;
+                ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+                if (!ok) break;
+                const float* slot = handover + (size_t)(blockIdx.x + 1) * (TILE_M * TILE_N);
+#pragma unroll
+                for (int i = 0; i < C::W; ++i) facc[i] = __ldcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local);
+                __syncwarp();
+                // this warp's bit back to zero for the next call
+                if (lane == 0) atomicAnd(handover_flags + blockIdx.x + 1, ~(1u << (warp - WARP_DRAIN0)));
+            }
             if (RES) {
                 // the residual of this warp's part of the tile (W tokens x 64 bytes) is asked into L2 now; the epilogue's
                 // loads then find it there
@@ -552,28 +567,13 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             if (BAL && gb > 0) {
                 // Balanced walk: the tile's earlier groups belong to the CTA before this one, which reaches
                 // them at the end of its range.  Hand this CTA's sums over: element (token t, channel n) at
-                // t * 128 + n of this CTA's slot, then the flag (release) once all eight drain warps have written.
+                // t * 128 + n of this CTA's slot, then this warp's bit of the slot's flag word (release).
                 float* slot = handover + (size_t)blockIdx.x * (TILE_M * TILE_N);
 #pragma unroll
                 for (int i = 0; i < C::W; ++i) __stcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local, facc[i]);
-                // the barrier orders the eight warps' stores before the one release below (cumulative at gpu scope)
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (warp == WARP_DRAIN0 && lane == 0) ptx::st_release_gpu_u32(handover_flags + blockIdx.x, 1u);
+                __syncwarp();
+                if (lane == 0) ptx::red_or_release_gpu_u32(handover_flags + blockIdx.x, 1u << (warp - WARP_DRAIN0));
                 continue;                       // the other CTA stores the tile
-            }
-            if (BAL && ge < G) {
-                // ... and this CTA holds the earlier groups of a tile whose later groups the next CTA summed
-                // long ago (they opened its range): wait for its flag (bounded), add its sums, clear the flag
-                if (warp == WARP_DRAIN0 && lane == 0) {
-                    if (!ptx::wait_flag_acquire_gpu(handover_flags + blockIdx.x + 1, 1u, abort_flag)) ok = false;
-                }
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (*abort_flag) { ok = false; break; }
-                const float* slot = handover + (size_t)(blockIdx.x + 1) * (TILE_M * TILE_N);
-#pragma unroll
-                for (int i = 0; i < C::W; ++i) facc[i] += __ldcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local);
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (warp == WARP_DRAIN0 && lane == 0) handover_flags[blockIdx.x + 1] = 0u;     // zero again for the next call
             }
             if (SPLIT) {
                 // every CTA of the cluster is past its last MMA: the activation rings are free and become
