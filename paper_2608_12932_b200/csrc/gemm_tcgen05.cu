@@ -462,8 +462,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 // start from those.  Fetched here and not after the last group they are off the tail that the launch ends with,
                 // and warp by warp (a flag bit each) they need no barrier of the CTA.  (4096 -> 24576 at 200 tokens 32.5 us, now
                 // 31.8; 12288 -> 4096 at 1024 with residual 70.5, now 69.1)
-                if (lane == 0 && !ptx::wait_bit_acquire_gpu(handover_flags + blockIdx.x + 1, 1u << (warp - WARP_DRAIN0), abort_flag)) ok = false;
-                ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+                ok = ptx::warp_wait_bit_acquire_gpu(handover_flags + blockIdx.x + 1, 1u << (warp - WARP_DRAIN0), abort_flag);
                 if (!ok) break;
                 const float* slot = handover + (size_t)(blockIdx.x + 1) * (TILE_M * TILE_N);
 #pragma unroll

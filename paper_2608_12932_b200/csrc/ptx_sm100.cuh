@@ -204,6 +204,15 @@ __device__ __forceinline__ bool wait_bit_acquire_gpu(const uint32_t* p, uint32_t
         __nanosleep(100);
     }
 }
+// The same for a whole warp, converged: lane 0 polls, and __syncwarp (a shuffle orders no memory) extends what it acquired
+// to the reads of the other lanes.
+__device__ __forceinline__ bool warp_wait_bit_acquire_gpu(const uint32_t* p, uint32_t mask, volatile uint32_t* abort_flag) {
+    bool ok = true;
+    if ((threadIdx.x & 31) == 0) ok = wait_bit_acquire_gpu(p, mask, abort_flag);
+    ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+    __syncwarp();
+    return ok;
+}
 
 // two floats rounded to bf16, the first in the low half
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {

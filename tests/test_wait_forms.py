@@ -1,0 +1,22 @@
+"""Source checks of how the kernels wait for one another, which no run can show: a hand-over that a warp acquires through one
+lane is ordered for its other lanes."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_12932_b200", "csrc")
+
+
+def code(name):
+    """A source file without its // comments."""
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_one_lane_acquires_go_through_the_warp_form():
+    """`lane == 0` polling with acquire orders memory for that lane alone: every kernel takes the form that ends in __syncwarp,
+    and that form does."""
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith(".cu"):
+            assert not re.search(r"(?<!warp_)wait_bit_acquire_gpu\(", code(name)), name
+    body = re.search(r"bool warp_wait_bit_acquire_gpu\([^)]*\) \{(.*?)\n\}", code("ptx_sm100.cuh"), re.S).group(1)
+    assert body.index("__shfl_sync") < body.index("__syncwarp();") < body.index("return")
