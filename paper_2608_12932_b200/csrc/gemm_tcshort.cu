@@ -496,31 +496,28 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             if (BAL && gb > 0) {
                 // Balanced walk: the tile's earlier groups belong to the CTA before this one, which reaches
                 // them at the end of its range.  Hand this CTA's sums over: element (token t, channel n) at
-                // t * 128 + n of this CTA's slot, then the flag (release) once all eight drain warps have written.
+                // t * 128 + n of this CTA's slot, then this warp's bit of the slot's flag word (release).  Warp by warp, because
+                // a barrier of the drain warps has no limit: after a time-out elsewhere the warps that gave up never reach it.
                 float* slot = handover + (size_t)blockIdx.x * (TILE_M * TILE_N);
 #pragma unroll
                 for (int i = 0; i < C::W; ++i) __stcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local, sum(i));
-                // the barrier orders the eight warps' stores before the one release below (cumulative at gpu scope)
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (warp == WARP_DRAIN0 && lane == 0) ptx::st_release_gpu_u32(handover_flags + blockIdx.x, 1u);
+                __syncwarp();
+                if (lane == 0) ptx::red_or_release_gpu_u32(handover_flags + blockIdx.x, 1u << (warp - WARP_DRAIN0));
                 continue;                       // the other CTA stores the tile
             }
             if (BAL && ge < G) {
                 // ... and this CTA holds the earlier groups of a tile whose later groups the next CTA summed
-                // long ago (they opened its range): wait for its flag (bounded), add its sums, clear the flag
-                if (warp == WARP_DRAIN0 && lane == 0) {
-                    if (!ptx::wait_flag_acquire_gpu(handover_flags + blockIdx.x + 1, 1u, abort_flag)) ok = false;
-                }
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (*abort_flag) { ok = false; break; }
+                // long ago (they opened its range): wait for this warp's bit (bounded), add its sums, clear the bit
+                ok = ptx::warp_wait_bit_acquire_gpu(handover_flags + blockIdx.x + 1, 1u << (warp - WARP_DRAIN0), abort_flag);
+                if (!ok) break;
                 const float* slot = handover + (size_t)(blockIdx.x + 1) * (TILE_M * TILE_N);
 #pragma unroll
                 for (int i = 0; i < C::W; i += 2) {
                     const float* p = slot + (size_t)(h * C::W + i) * TILE_N + n_local;
                     facc[i / 2] = ptx::add2(facc[i / 2], ptx::pack2(__float_as_uint(__ldcg(p)), __float_as_uint(__ldcg(p + TILE_N))));
                 }
-                ptx::named_bar_sync(2, NUM_DRAIN_WARPS * 32);
-                if (warp == WARP_DRAIN0 && lane == 0) handover_flags[blockIdx.x + 1] = 0u;     // zero again for the next call
+                __syncwarp();
+                if (lane == 0) atomicAnd(handover_flags + blockIdx.x + 1, ~(1u << (warp - WARP_DRAIN0)));     // zero again for the next call
             }
             if (SPLIT) {
                 // every CTA of the cluster is past its last MMA: the rings are free and become

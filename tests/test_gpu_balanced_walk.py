@@ -15,7 +15,8 @@ from tests.gpu_util import DeviceLayer, bits, t_u16
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,K,N,tile", [(849, 3200, 4096, 128), (849, 2944, 4096, 208)])
+@pytest.mark.parametrize("M,K,N,tile", [(849, 3200, 4096, 128), (849, 2944, 4096, 208), (20, 2688, 19200, 64), (32, 3200, 19200, 64),
+                                        (40, 3200, 19200, 64), (64, 3456, 19200, 64), (588, 3200, 2048, 64)])
 def test_tiles_shared_by_neighbours(M, K, N, tile):
     plan = B.w4a8_plan(M, N, K)
     assert plan["family"] == B.PATH_TCGEN05 and plan["tile_m"] == tile and plan["balanced"] == 1

@@ -1,5 +1,5 @@
 """Source checks of how the kernels wait for one another, which no run can show: a hand-over that a warp acquires through one
-lane is ordered for its other lanes."""
+lane is ordered for its other lanes, and no warp waits without a limit for warps that may have given up."""
 import os
 import re
 
@@ -20,3 +20,11 @@ def test_one_lane_acquires_go_through_the_warp_form():
             assert not re.search(r"(?<!warp_)wait_bit_acquire_gpu\(", code(name)), name
     body = re.search(r"bool warp_wait_bit_acquire_gpu\([^)]*\) \{(.*?)\n\}", code("ptx_sm100.cuh"), re.S).group(1)
     assert body.index("__shfl_sync") < body.index("__syncwarp();") < body.index("return")
+
+
+def test_no_barrier_inside_the_roles_of_the_tensor_core_kernels():
+    """Their roles leave their loops one by one when a wait runs out, so a barrier among some warps could wait for good: the only
+    block barriers are the two that every thread reaches, after the set-up and before tensor memory is given back."""
+    for name in ("gemm_tcgen05.cu", "gemm_tcshort.cu"):
+        text = code(name)
+        assert "named_bar_sync" not in text and "bar.sync" not in text and text.count("__syncthreads()") == 2, name
