@@ -1,6 +1,6 @@
 """GPU parity of the short-tile tensor-core kernel (64-row token tiles, cut to 32 columns up to 32 tokens) where it can go
 wrong: odd group counts against its two-group steps, one group, both tile widths and their edges, K splits with uneven
-shares, tiles shared by neighbouring CTAs, and the extreme partials that its accumulator bias has to cover.  Partials D
+shares, more tiles than SMs, and the extreme partials that its accumulator bias has to cover.  Partials D
 bit-exact, output within the band of the linear layer, against the CPU oracle."""
 import numpy as np
 import pytest
@@ -31,8 +31,10 @@ def test_group_counts_and_tile_edges(K, N):
     case = wl.make_layer(K, N, 60 + K // 128, 130)
     layer = DeviceLayer(case, 130)
     for M in (1, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129):
-        if B.w4a8_plan(max(M, 17), N, K)["tile_m"] == 64:
-            check(case, layer, M)
+        if M > 64:                                          # (up to 64 tokens no taller tile is considered)
+            plan = B.w4a8_plan(M, N, K)
+            assert plan["family"] == B.PATH_TCGEN05 and plan["tile_m"] == 64
+        check(case, layer, M)
 
 
 @pytest.mark.parametrize("M,K,N", [(20, 3200, 512), (40, 3200, 512), (64, 3456, 512), (100, 3456, 256)])
@@ -48,13 +50,13 @@ def test_uneven_k_split(M, K, N):
 
 
 @pytest.mark.parametrize("M,K,N", [(20, 1152, 24576), (40, 1152, 24576), (300, 1152, 4352)])
-def test_tiles_shared_by_neighbours(M, K, N):
-    """More tiles than SMs, nine groups each: ranges start and end inside tiles at odd and even groups; the hand-over flags
-    are back at zero for the second call."""
+def test_more_tiles_than_sms(M, K, N):
+    """More tiles than SMs, nine groups each, as whole tiles: rings and accumulator buffers run on from one tile to the next
+    behind a lone last group.  (Tiles shared by neighbouring CTAs: test_gpu_balanced_walk.py.)"""
     case = wl.make_layer(K, N, 72, M)
     layer = DeviceLayer(case, M)
     plan = B.w4a8_plan(M, N, K)
-    assert plan["tile_m"] == 64
+    assert plan["tile_m"] == 64 and plan["k_slices"] == 1 and plan["balanced"] == 0
     y1 = check(case, layer, M, debug=False)
     assert np.array_equal(y1, check(case, layer, M, debug=False))
 
