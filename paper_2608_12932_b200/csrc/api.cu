@@ -155,21 +155,28 @@ w4a8_status w4a8_unpack_weights(const void* packed, int N, int K, int group,
                ? W4A8_OK : W4A8_ERR_CUDA;
 }
 
-w4a8_status w4a8_quantize_act(const void* x_bf16, int M, int K, int group,
-                              int8_t* qa, uint16_t* sa, int32_t* asum, void* stream) {
+// x_copy: null, or a buffer that receives x
+static w4a8_status quantize_impl(const void* x_bf16, void* x_copy, int M, int K, int group,
+                                 int8_t* qa, uint16_t* sa, int32_t* asum, void* stream) {
     if (group != GROUP || K <= 0 || K % GROUP != 0 || M < 0) return W4A8_ERR_SHAPE;
     if (M == 0) return W4A8_OK;
     if (!x_bf16 || !qa || !sa || !asum) return W4A8_ERR_NULL;
     if (!aligned(x_bf16, 16) || !aligned(qa, 16) || !aligned(sa, 2) || !aligned(asum, 4)) return W4A8_ERR_ALIGN;
     w4a8_status a = arch_check();
     if (a != W4A8_OK) return a;
-    return launch_quantize_act(x_bf16, M, K, qa, sa, asum, static_cast<cudaStream_t>(stream)) == cudaSuccess
+    return launch_quantize_act(x_bf16, M, K, qa, sa, asum, static_cast<cudaStream_t>(stream), x_copy) == cudaSuccess
                ? W4A8_OK : W4A8_ERR_CUDA;
 }
 
+w4a8_status w4a8_quantize_act(const void* x_bf16, int M, int K, int group,
+                              int8_t* qa, uint16_t* sa, int32_t* asum, void* stream) {
+    return quantize_impl(x_bf16, nullptr, M, K, group, qa, sa, asum, stream);
+}
+
+// y_copy: null, or a second buffer that receives y (the strip and cluster kernels only)
 static w4a8_status gemm_impl(w4a8_path path,
                              const int8_t* qa, const uint16_t* sa, const int32_t* asum,
-                             const void* packed_w, void* y_bf16, const void* residual,
+                             const void* packed_w, void* y_bf16, const void* residual, void* y_copy,
                              int M, int N, int K, int group,
                              void* workspace, size_t workspace_bytes,
                              int32_t* debug_partials, void* stream) {
@@ -197,9 +204,9 @@ static w4a8_status gemm_impl(w4a8_path path,
         e = launch_gemm_splitk(qa, sa, asum, packed_w, y_bf16, M, N, K, workspace,
                                reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + WS_SHARED_OFF), debug_partials, st);
     else if (path == W4A8_PATH_STRIP || (path == W4A8_PATH_AUTO && auto_takes_strip(M, N, K)))
-        e = launch_gemm_strip(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
+        e = launch_gemm_strip(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st, y_copy);
     else if (path == W4A8_PATH_SPLITK || (path == W4A8_PATH_AUTO && !small_m_prefers_tcgen05(M, N, K, device_sm_count())))
-        e = launch_gemm_cluster(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
+        e = launch_gemm_cluster(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st, y_copy);
     else
         e = launch_gemm_tcgen05(qa, sa, asum, packed_w, y_bf16, residual, M, N, K, workspace, debug_partials, st);
     return e == cudaSuccess ? W4A8_OK : W4A8_ERR_CUDA;
@@ -211,14 +218,14 @@ w4a8_status w4a8_gemm_path(w4a8_path path,
                            int M, int N, int K, int group,
                            void* workspace, size_t workspace_bytes,
                            int32_t* debug_partials, void* stream) {
-    return gemm_impl(path, qa, sa, asum, packed_w, y_bf16, nullptr, M, N, K, group, workspace, workspace_bytes, debug_partials, stream);
+    return gemm_impl(path, qa, sa, asum, packed_w, y_bf16, nullptr, nullptr, M, N, K, group, workspace, workspace_bytes, debug_partials, stream);
 }
 
 w4a8_status w4a8_gemm_residual(w4a8_path path, const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed_w,
                                const void* residual_bf16, void* y_bf16, int M, int N, int K, int group,
                                void* workspace, size_t workspace_bytes, void* stream) {
     if (M > 0 && !residual_bf16) return W4A8_ERR_NULL;
-    return gemm_impl(path, qa, sa, asum, packed_w, y_bf16, residual_bf16, M, N, K, group, workspace, workspace_bytes, nullptr, stream);
+    return gemm_impl(path, qa, sa, asum, packed_w, y_bf16, residual_bf16, nullptr, M, N, K, group, workspace, workspace_bytes, nullptr, stream);
 }
 
 w4a8_status w4a8_silu_mul_quantize(const void* y_gate_up_bf16, int M, int I, int group, void* h_bf16,
@@ -372,19 +379,27 @@ w4a8_status w4a8_gemm(const int8_t* qa, const uint16_t* sa, const int32_t* asum,
                           workspace, workspace_bytes, debug_partials, stream);
 }
 
-w4a8_status w4a8_linear(const void* x_bf16, const void* packed_w, void* y_bf16,
-                        int M, int N, int K, int group,
-                        int8_t* qa, uint16_t* sa, int32_t* asum,
-                        void* workspace, size_t workspace_bytes, void* stream) {
+static w4a8_status linear_impl(const void* x_bf16, void* x_copy, const void* packed_w, void* y_bf16, void* y_copy,
+                               int M, int N, int K, int group,
+                               int8_t* qa, uint16_t* sa, int32_t* asum,
+                               void* workspace, size_t workspace_bytes, void* stream) {
     if (!shape_ok(N, K, group) || M < 0) return W4A8_ERR_SHAPE;
     if (M == 0) return W4A8_OK;
     // everything the second call would refuse is refused before the first one is enqueued
     if (!x_bf16 || !qa || !sa || !asum || !packed_w || !y_bf16 || !workspace) return W4A8_ERR_NULL;
     if (!aligned(packed_w, 128) || !aligned(y_bf16, 16) || !aligned(workspace, 256)) return W4A8_ERR_ALIGN;
     if (workspace_bytes < w4a8_workspace_bytes(M, N, K, group)) return W4A8_ERR_WORKSPACE;
-    w4a8_status s = w4a8_quantize_act(x_bf16, M, K, group, qa, sa, asum, stream);
+    w4a8_status s = quantize_impl(x_bf16, x_copy, M, K, group, qa, sa, asum, stream);
     if (s != W4A8_OK) return s;
-    return w4a8_gemm(qa, sa, asum, packed_w, y_bf16, M, N, K, group, workspace, workspace_bytes, nullptr, stream);
+    return gemm_impl(W4A8_PATH_AUTO, qa, sa, asum, packed_w, y_bf16, nullptr, y_copy, M, N, K, group, workspace,
+                     workspace_bytes, nullptr, stream);
+}
+
+w4a8_status w4a8_linear(const void* x_bf16, const void* packed_w, void* y_bf16,
+                        int M, int N, int K, int group,
+                        int8_t* qa, uint16_t* sa, int32_t* asum,
+                        void* workspace, size_t workspace_bytes, void* stream) {
+    return linear_impl(x_bf16, nullptr, packed_w, y_bf16, nullptr, M, N, K, group, qa, sa, asum, workspace, workspace_bytes, stream);
 }
 
 w4a8_status w4a8_linear_host(const void* x_host_bf16, void* y_host_bf16,
@@ -400,22 +415,21 @@ w4a8_status w4a8_linear_host(const void* x_host_bf16, void* y_host_bf16,
         return W4A8_ERR_ALIGN;
     if (workspace_bytes < w4a8_workspace_bytes(M, N, K, group)) return W4A8_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // Small requests in pinned memory: the quantiser reads x where it is, and the kernels that store y in plain 16-byte
-    // pieces write it where it goes.  A copy engine costs the stream two hand-overs per copy, several microseconds, to
-    // move what the kernels themselves move in one or two.
-    const void* x_at = x_dev;
-    void* y_at = y_dev;
+    // Small requests in pinned memory: the quantiser reads x where it is, and the kernels that store y in plain 8- and
+    // 16-byte pieces write it where it goes as well.  A copy engine costs the stream two hand-overs per copy, several
+    // microseconds, to move what the kernels themselves move in one or two.  x_dev and y_dev are filled either way.
+    const void* x_pinned = nullptr;
+    void* y_pinned = nullptr;
     if ((size_t)M * K * 2 <= HOST_DIRECT_MAX_BYTES) {
-        if (void* p = pinned_device_address(x_host_bf16)) x_at = p;
-        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K)) {
-            if (void* p = pinned_device_address(y_host_bf16)) y_at = p;
-        }
+        x_pinned = pinned_device_address(x_host_bf16);
+        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K)) y_pinned = pinned_device_address(y_host_bf16);
     }
-    if (x_at == x_dev && cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    if (!x_pinned && cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return W4A8_ERR_CUDA;
-    w4a8_status s = w4a8_linear(x_at, packed_w, y_at, M, N, K, group, qa, sa, asum, workspace, workspace_bytes, stream);
+    w4a8_status s = linear_impl(x_pinned ? x_pinned : x_dev, x_pinned ? x_dev : nullptr, packed_w, y_dev, y_pinned, M, N, K, group,
+                                qa, sa, asum, workspace, workspace_bytes, stream);
     if (s != W4A8_OK) return s;
-    if (y_at == y_dev && cudaMemcpyAsync(y_host_bf16, y_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    if (!y_pinned && cudaMemcpyAsync(y_host_bf16, y_dev, (size_t)M * N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return W4A8_ERR_CUDA;
     return W4A8_OK;
 }

@@ -76,8 +76,8 @@ template <int MB, int MINB, int RB>
 __global__ void __launch_bounds__(CL_THREADS, MINB)
 gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmap_qa, const uint16_t* __restrict__ sa,
                     const int32_t* __restrict__ asum, const uint8_t* __restrict__ packed,
-                    __nv_bfloat16* y, const __nv_bfloat16* residual, int M, int N, int K, int S, int ng_max, int stages,
-                    uint32_t* __restrict__ status, int32_t* __restrict__ debug_partials) {
+                    __nv_bfloat16* y, const __nv_bfloat16* residual, __nv_bfloat16* y_copy, int M, int N, int K, int S,
+                    int ng_max, int stages, uint32_t* __restrict__ status, int32_t* __restrict__ debug_partials) {
     ptx::pdl_launch_dependents();
     ptx::cluster_arrive_relaxed();     // "this CTA runs": peers wait for it before they write into it
     extern __shared__ uint8_t smem_raw[];
@@ -356,13 +356,14 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmap_qa, const uint16_t*
             o.x = *reinterpret_cast<uint32_t*>(&o01);
             o.y = *reinterpret_cast<uint32_t*>(&o23);
             *reinterpret_cast<uint2*>(y + (size_t)m * N + (size_t)ntile * TILE_N + nn) = o;
+            if (y_copy) *reinterpret_cast<uint2*>(y_copy + (size_t)m * N + (size_t)ntile * TILE_N + nn) = o;
         }
     }
 }
 
 template <int MB, int MINB, int RB>
 cudaError_t launch_mb(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y, const void* residual,
-                      int M, int N, int K, int S, void* workspace, int32_t* debug_partials, cudaStream_t stream) {
+                      void* y_copy, int M, int N, int K, int S, void* workspace, int32_t* debug_partials, cudaStream_t stream) {
     const int G = K / GROUP;
     const int ng_max = (G + S - 1) / S;
     // shared-memory budget per CTA: a launch of at most one wave leaves room for the next launch's
@@ -419,7 +420,8 @@ cudaError_t launch_mb(const int8_t* qa, const uint16_t* sa, const int32_t* asum,
     cfg.numAttrs = 3;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<MB, MINB, RB>, tmap, sa, asum, static_cast<const uint8_t*>(packed),
-                              static_cast<__nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(residual), M, N, K, S, ng_max, stages,
+                              static_cast<__nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(residual),
+                              static_cast<__nv_bfloat16*>(y_copy), M, N, K, S, ng_max, stages,
                               reinterpret_cast<uint32_t*>(ws + WS_STATUS_OFF), debug_partials);
 }
 }  // namespace
@@ -445,23 +447,23 @@ int cluster_num_slices(int M, int N, int K) {
 
 cudaError_t launch_gemm_cluster(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                                 void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
-                                cudaStream_t stream) {
+                                cudaStream_t stream, void* y_copy) {
     const int S = cluster_num_slices(M, N, K);
     if (M <= 8) {
         // two launches co-resident.  Four warp sets (each warp two blocks of 16 rows) when a slice is
         // long enough to give every set at least two groups: more groups in flight per CTA and the
         // activation fragments are loaded once for both blocks.
         const int ng_max = (K / GROUP + S - 1) / S;
-        if (ng_max >= 8) return launch_mb<1, 2, 2>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
-        return launch_mb<1, 2, 1>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
+        if (ng_max >= 8) return launch_mb<1, 2, 2>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
+        return launch_mb<1, 2, 1>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
     }
     if (M <= 16) {
         if ((N / TILE_N) * S > device_sm_count())
-            return launch_mb<2, 2, 1>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
-        return launch_mb<2, 1, 1>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
+            return launch_mb<2, 2, 1>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
+        return launch_mb<2, 1, 1>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
     }
-    if (M <= 32) return launch_mb<4, 1, 1>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
-    return launch_mb<8, 1, 1>(qa, sa, asum, packed, y, residual, M, N, K, S, workspace, debug_partials, stream);
+    if (M <= 32) return launch_mb<4, 1, 1>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
+    return launch_mb<8, 1, 1>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, S, workspace, debug_partials, stream);
 }
 
 }  // namespace w4a8

@@ -178,6 +178,7 @@ struct StripArgs {
     const int32_t* asum;
     const uint8_t* packed;
     __nv_bfloat16* y;
+    __nv_bfloat16* y_copy;   // null, or a second place for y (the plain form only)
     int M, N, K;
     int stages;              // ring length
     int pre;                 // ring slots whose weights are requested before griddepcontrol.wait (the rest: L2 prefetch).
@@ -676,6 +677,7 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
                     const int m = c / CPR, col = c - m * CPR;
                     const uint4 v = ptx::lds128(ystage + m * YPITCH + col * 16);
                     *reinterpret_cast<uint4*>(a.y + (size_t)m * a.N + (size_t)strip * R + col * 8) = v;
+                    if (a.y_copy) *reinterpret_cast<uint4*>(a.y_copy + (size_t)m * a.N + (size_t)strip * R + col * 8) = v;
                 }
                 __syncwarp();
             }
@@ -800,8 +802,8 @@ struct FuseOut {
 
 template <int MB, int RBLK, bool DEBUG, int FUSE>
 cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
-                         const void* residual, int M, int N, int K, int ctas, void* workspace, int32_t* debug_partials,
-                         const FuseOut* fuse, cudaStream_t stream) {
+                         const void* residual, void* y_copy, int M, int N, int K, int ctas, void* workspace,
+                         int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
     constexpr int R = 16 * RBLK, GS = ST_UNITS / RBLK, MP = 8 * MB;
     const int G = K / GROUP;
     const bool fp32_stage = FUSE == 3;
@@ -842,6 +844,7 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     a.asum = asum;
     a.packed = static_cast<const uint8_t*>(packed);
     a.y = static_cast<__nv_bfloat16*>(y);
+    a.y_copy = static_cast<__nv_bfloat16*>(y_copy);
     a.M = M; a.N = N; a.K = K;
     a.stages = stages;
     a.pre = stages;
@@ -882,23 +885,23 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
 
 template <int MB, int RBLK>
 cudaError_t launch_strip_dbg(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
-                             const void* residual, int M, int N, int K, int ctas, void* workspace, int32_t* debug_partials, const FuseOut* fuse,
-                             cudaStream_t stream) {
+                             const void* residual, void* y_copy, int M, int N, int K, int ctas, void* workspace,
+                             int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
     if (fuse) {
         // two token blocks always run on 32-row strips (strip_plan): the other widths are not built in the fused form
         if constexpr (MB == 2 && RBLK != 2) return cudaErrorInvalidConfiguration;
         else if (fuse->one_kernel)
-            return launch_strip<MB, RBLK, false, 1>(qa, sa, asum, packed, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
+            return launch_strip<MB, RBLK, false, 1>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
         else
-            return launch_strip<MB, RBLK, false, 2>(qa, sa, asum, packed, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
+            return launch_strip<MB, RBLK, false, 2>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
     }
     if (residual) {                                      // its own instantiation: the plain kernel's epilogue stays as small as it was
         if constexpr (MB == 2 && RBLK != 2) return cudaErrorInvalidConfiguration;
-        else return launch_strip<MB, RBLK, false, 3>(qa, sa, asum, packed, y, residual, M, N, K, ctas, workspace, nullptr, nullptr, stream);
+        else return launch_strip<MB, RBLK, false, 3>(qa, sa, asum, packed, y, residual, nullptr, M, N, K, ctas, workspace, nullptr, nullptr, stream);
     }
     if (debug_partials)
-        return launch_strip<MB, RBLK, true, 0>(qa, sa, asum, packed, y, nullptr, M, N, K, ctas, workspace, debug_partials, nullptr, stream);
-    return launch_strip<MB, RBLK, false, 0>(qa, sa, asum, packed, y, nullptr, M, N, K, ctas, workspace, nullptr, nullptr, stream);
+        return launch_strip<MB, RBLK, true, 0>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, debug_partials, nullptr, stream);
+    return launch_strip<MB, RBLK, false, 0>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, nullptr, nullptr, stream);
 }
 
 }  // namespace
@@ -954,12 +957,12 @@ void strip_plan(int M, int N, int K, int* strip_rows, int* ctas) {
 
 namespace {
 cudaError_t strip_dispatch(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
-                           void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials, const FuseOut* fuse,
-                           cudaStream_t stream) {
+                           void* y, const void* residual, void* y_copy, int M, int N, int K, void* workspace,
+                           int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
     int R = 0, ctas = 0;
     strip_plan(M, N, K, &R, &ctas);
 #define W4A8_STRIP_CASE(MBV, RBV) \
-    return launch_strip_dbg<MBV, RBV>(qa, sa, asum, packed, y, residual, M, N, K, ctas, workspace, debug_partials, fuse, stream)
+    return launch_strip_dbg<MBV, RBV>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, ctas, workspace, debug_partials, fuse, stream)
     if (M <= 8) {
         if (R == 128) W4A8_STRIP_CASE(1, 8);
         if (R == 64) W4A8_STRIP_CASE(1, 4);
@@ -976,8 +979,8 @@ cudaError_t strip_dispatch(const int8_t* qa, const uint16_t* sa, const int32_t* 
 
 cudaError_t launch_gemm_strip(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                               void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
-                              cudaStream_t stream) {
-    return strip_dispatch(qa, sa, asum, packed, y, residual, M, N, K, workspace, debug_partials, nullptr, stream);
+                              cudaStream_t stream, void* y_copy) {
+    return strip_dispatch(qa, sa, asum, packed, y, residual, y_copy, M, N, K, workspace, debug_partials, nullptr, stream);
 }
 
 // The fused gate+up form: packed = the 2 I = N channels in runs of eight gate / eight up; outputs h [M, I] bf16 and the
@@ -986,7 +989,7 @@ cudaError_t launch_gemm_strip_gate_up(const int8_t* qa, const uint16_t* sa, cons
                                       int M, int N, int K, void* h, int8_t* qa_h, uint16_t* sa_h, int32_t* asum_h,
                                       bool one_kernel, void* workspace, cudaStream_t stream) {
     const FuseOut f = {h, qa_h, sa_h, asum_h, one_kernel};
-    return strip_dispatch(qa, sa, asum, packed, nullptr, nullptr, M, N, K, workspace, nullptr, &f, stream);
+    return strip_dispatch(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, workspace, nullptr, &f, stream);
 }
 
 }  // namespace w4a8

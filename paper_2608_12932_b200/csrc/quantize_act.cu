@@ -70,7 +70,9 @@ __device__ __forceinline__ uint32_t quant4_fast(uint32_t lo_pair, uint32_t hi_pa
 // alternate between eight gate channels and the eight up channels of the same indices; the row that is quantised
 // is h = bf16(SiLU(gate) * up), K values, computed chunk by chunk as it is loaded (Sec. 3.5: the element-wise
 // step merged into its consumer) and, if h_out is given, also stored.
-template <int QA_THREADS, int QA_CACHE, bool FAST, bool SILU>
+//
+// COPY: the row itself is also stored, in h_out (a form of its own: the plain kernel stays as it is).
+template <int QA_THREADS, int QA_CACHE, bool FAST, bool SILU, bool COPY>
 __global__ void __launch_bounds__(QA_THREADS, QA_THREADS == 256 ? (QA_CACHE == 2 ? 8 : 5) : (QA_THREADS == 512 ? 3 : 1))
 quantize_act_kernel(const uint4* __restrict__ x, int K, uint2* __restrict__ qa,
                     uint16_t* __restrict__ sa, int32_t* __restrict__ asum, uint4* __restrict__ h_out) {
@@ -142,7 +144,7 @@ quantize_act_kernel(const uint4* __restrict__ x, int K, uint2* __restrict__ qa,
             if (worst > 0.5f - 0.0001220703125f) o = quant8(v, s, sum);      // 2^-13: a possible tie in this chunk
         }
         qr[c] = o;
-        if (SILU && h_out) h_out[(size_t)m * chunks + c] = v;
+        if (COPY || (SILU && h_out)) h_out[(size_t)m * chunks + c] = v;
         sum += __shfl_xor_sync(seg_mask, sum, 8);
         sum += __shfl_xor_sync(seg_mask, sum, 4);
         sum += __shfl_xor_sync(seg_mask, sum, 2);
@@ -254,7 +256,7 @@ cudaError_t launch_silu_cluster(cudaLaunchConfig_t cfg, int M, int C, const uint
     cfg.blockDim = dim3(T, 1, 1);
     return cudaLaunchKernelEx(&cfg, silu_quantize_cluster_kernel<T, R>, x, K, C, qa, sa, asum, h);
 }
-template <bool SILU>
+template <bool SILU, bool COPY = false>
 cudaError_t launch_quantize(const void* x, int M, int K, int8_t* qa, uint16_t* sa, int32_t* asum, void* h_out,
                             cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
@@ -288,17 +290,18 @@ cudaError_t launch_quantize(const void* x, int M, int K, int8_t* qa, uint16_t* s
         }
     }
     if (threads == 1024)
-        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<1024, QA_CACHE_CHUNKS / 1024, false, SILU>, xp, K, qp, sa, asum, hp);
+        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<1024, QA_CACHE_CHUNKS / 1024, false, SILU, COPY>, xp, K, qp, sa, asum, hp);
     if (threads == 512)
-        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<512, QA_CACHE_CHUNKS / 512, false, SILU>, xp, K, qp, sa, asum, hp);
+        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<512, QA_CACHE_CHUNKS / 512, false, SILU, COPY>, xp, K, qp, sa, asum, hp);
     if (K <= 256 * 2 * 8)                                    // rows of up to 4096: two chunks per thread, eight rows per SM
-        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<256, 2, true, SILU>, xp, K, qp, sa, asum, hp);
-    return cudaLaunchKernelEx(&cfg, quantize_act_kernel<256, QA_CACHE_CHUNKS / 256, true, SILU>, xp, K, qp, sa, asum, hp);
+        return cudaLaunchKernelEx(&cfg, quantize_act_kernel<256, 2, true, SILU, COPY>, xp, K, qp, sa, asum, hp);
+    return cudaLaunchKernelEx(&cfg, quantize_act_kernel<256, QA_CACHE_CHUNKS / 256, true, SILU, COPY>, xp, K, qp, sa, asum, hp);
 }
 }  // namespace
 
 cudaError_t launch_quantize_act(const void* x, int M, int K, int8_t* qa, uint16_t* sa, int32_t* asum,
-                                cudaStream_t stream) {
+                                cudaStream_t stream, void* x_copy) {
+    if (x_copy) return launch_quantize<false, true>(x, M, K, qa, sa, asum, x_copy, stream);
     return launch_quantize<false>(x, M, K, qa, sa, asum, nullptr, stream);
 }
 

@@ -70,8 +70,9 @@ cudaError_t make_y_tensor_map(CUtensorMap* out, void* y, int M, int N);
 cudaError_t make_strip_weight_maps(CUtensorMap* nib, CUtensorMap* scale, CUtensorMap* zero, const void* packed,
                                    int N, int K, int R, int GS);
 cudaError_t make_qa_group_map(CUtensorMap* out, const int8_t* qa, int M, int K, int box_rows, int box_groups);
+// x_copy (bf16 [M, K], 16-byte aligned) may be null; otherwise it receives x
 cudaError_t launch_quantize_act(const void* x, int M, int K, int8_t* qa, uint16_t* sa, int32_t* asum,
-                                cudaStream_t stream);
+                                cudaStream_t stream, void* x_copy = nullptr);
 // h = bf16(SiLU(gate) * up) of a chunk-interleaved gate+up output y [M, 2 I], quantised like an activation row;
 // h_out (bf16 [M, I]) may be null
 cudaError_t launch_silu_mul_quantize(const void* y_gate_up, int M, int I, void* h_out, int8_t* qa, uint16_t* sa,
@@ -92,9 +93,10 @@ constexpr int STRIP_SLOT_BYTES = TILE_N * STRIP_MAX_M * 8;  // one strip's fp32 
 static_assert(WS_HEADER_BYTES + STRIP_MAX_CTAS * STRIP_SLOT_BYTES == W4A8_WORKSPACE_ZEROED_BYTES, "strip slots fill the zeroed part");
 bool strip_supported(int M, int N, int K);
 void strip_plan(int M, int N, int K, int* strip_rows, int* ctas);
+// y_copy (here and in the cluster kernel's plain form): null, or a second bf16 [M,N] that receives y, 16-byte aligned
 cudaError_t launch_gemm_strip(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                               void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
-                              cudaStream_t stream);
+                              cudaStream_t stream, void* y_copy = nullptr);
 // streaming prefill: rotary embedding of pre-rotation cached keys at shifted positions; the streaming attention mask
 cudaError_t launch_rope_shifted_keys(const void* k_pre, const int32_t* pos, int delta, int T, int H, int D, double base,
                                      void* k_rot, cudaStream_t stream);
@@ -116,7 +118,7 @@ int cluster_num_slices(int M, int N, int K);
 // residual: null, or bf16 [M,N] added to the projection before the one rounding (may be y itself)
 cudaError_t launch_gemm_cluster(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                                 void* y, const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
-                                cudaStream_t stream);
+                                cudaStream_t stream, void* y_copy = nullptr);
 cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
                                 const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials,
                                 cudaStream_t stream);

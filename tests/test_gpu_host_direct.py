@@ -26,3 +26,22 @@ def test_equals_the_device_path(M, K, N, pin_x, pin_y):
         torch.cuda.synchronize()
         assert np.array_equal(y.view(torch.int16).numpy().view(np.uint16), want)
         y.fill_(float("nan"))
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 256, 256), (8, 4096, 6144), (16, 1024, 384), (12, 1024, 6144), (40, 1024, 512), (3, 16384, 128)])
+def test_new_inputs_in_the_same_buffers_and_the_device_copies(M, K, N):
+    """Every call reads what the pinned buffer holds at that time, and leaves x and y in the device staging buffers too."""
+    case = wl.make_layer(K, N, 90 + M, 3 * M)
+    layer = DeviceLayer(case, M)
+    linear = B.HostLinear(M, N, K, layer.packed, layer.ws)
+    linear.x_dev.fill_(7.0), linear.y_dev.fill_(7.0)
+    x = torch.empty((M, K), dtype=torch.bfloat16).pin_memory()
+    y = torch.empty((M, N), dtype=torch.bfloat16).pin_memory()
+    for i in range(3):
+        x_bits = case["x"][i * M:(i + 1) * M]
+        want = bits(B.w4a8_linear(t_u16(x_bits, torch.bfloat16), layer.packed, N, layer.ws))
+        x.view(torch.int16).copy_(torch.from_numpy(x_bits.view(np.int16)))
+        linear(x, y)
+        torch.cuda.synchronize()
+        assert np.array_equal(y.view(torch.int16).numpy().view(np.uint16), want)
+        assert np.array_equal(bits(linear.x_dev), x_bits) and np.array_equal(bits(linear.y_dev), want)
