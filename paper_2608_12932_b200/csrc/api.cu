@@ -1,6 +1,7 @@
 // extern "C" boundary of libw4a8: argument validation, dispatch by M, status codes.
 // Every step of the path runs in the CUDA kernels; nothing here touches the data.
 #include <cuda_runtime.h>
+#include "host_range.h"
 #include "w4a8_internal.cuh"
 
 using namespace w4a8;
@@ -73,15 +74,17 @@ bool takes_tcgen05(int M, int N, int K) {
     return !auto_takes_strip(M, N, K) && small_m_prefers_tcgen05(M, N, K, device_sm_count());
 }
 
-// The device's address of a buffer in pinned host memory, if it has one and a kernel can use 16-byte accesses there.
+// The device's address of a buffer in pinned host memory, or null if a kernel cannot use it there.
 constexpr size_t HOST_DIRECT_MAX_BYTES = 512 * 1024;
-void* pinned_device_address(const void* p) {
+void* pinned_device_address(const void* p, size_t bytes) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    return a.type == cudaMemoryTypeHost && aligned(a.devicePointer, 16) ? a.devicePointer : nullptr;
+    HostMemory m = {a.type == cudaMemoryTypeHost, a.devicePointer, 0, 0};
+    if (!m.pinned || !host_range_of(p, &m.start, &m.size)) return nullptr;
+    return in_place_address(m, p, bytes);
 }
 
 size_t slices_bytes(int M, int N, int K) {
@@ -421,8 +424,9 @@ w4a8_status w4a8_linear_host(const void* x_host_bf16, void* y_host_bf16,
     const void* x_pinned = nullptr;
     void* y_pinned = nullptr;
     if ((size_t)M * K * 2 <= HOST_DIRECT_MAX_BYTES) {
-        x_pinned = pinned_device_address(x_host_bf16);
-        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K)) y_pinned = pinned_device_address(y_host_bf16);
+        x_pinned = pinned_device_address(x_host_bf16, (size_t)M * K * 2);
+        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K))
+            y_pinned = pinned_device_address(y_host_bf16, (size_t)M * N * 2);
     }
     if (!x_pinned && cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return W4A8_ERR_CUDA;

@@ -1,6 +1,6 @@
-// Host-side construction of the TMA tensor map over the int8 activations qa[M,K]:
-// tiles of 128 k (one quantisation group, 128 bytes) x `box_rows` tokens, 128-byte swizzle,
-// rows past M read as zeros.  The driver entry point is resolved through the runtime so the
+// Calls of the driver's API: construction of the TMA tensor maps, and the range of a host buffer.
+// The map over the int8 activations qa[M,K]: tiles of 128 k (one quantisation group, 128 bytes) x `box_rows` tokens, 128-byte swizzle,
+// rows past M read as zeros.  The driver entry points are resolved through the runtime so the
 // library carries no link-time dependency on libcuda.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -25,6 +25,8 @@ EncodeTiledFn encode_tiled_fn() {
     }
     return fn;
 }
+
+typedef CUresult (*PointerAttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
 
 // Encoding a map costs the host about a microsecond and depends only on the pointer and the shape, not on
 // the memory's contents: the maps of the small-M kernel (three per call) are kept in a small table.
@@ -61,6 +63,25 @@ MapCache& map_cache() {
     return c;
 }
 }  // namespace
+
+bool host_range_of(const void* p, uint64_t* start, uint64_t* size) {
+    static const PointerAttributesFn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool found = cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &q) == cudaSuccess &&
+                           q == cudaDriverEntryPointSuccess;
+        return found ? reinterpret_cast<PointerAttributesFn>(f) : nullptr;
+    }();
+    if (!get) return false;
+    CUpointer_attribute which[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    CUdeviceptr at = 0;
+    size_t bytes = 0;
+    void* out[2] = {&at, &bytes};
+    if (get(2, which, out, (CUdeviceptr)reinterpret_cast<uintptr_t>(p)) != CUDA_SUCCESS) return false;
+    *start = at;
+    *size = bytes;
+    return bytes > 0;
+}
 
 // Views of the packed weights for the strip kernel: a strip is R < 128 consecutive rows of a 128-channel tile
 // (whole tiles are fetched with plain bulk copies and need no map).

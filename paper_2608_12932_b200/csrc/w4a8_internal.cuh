@@ -113,6 +113,8 @@ cudaError_t make_x_half_group_map(CUtensorMap* out, const void* x, int M, int K,
 cudaError_t launch_gemm_strip_gate_up(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed,
                                       int M, int N, int K, void* h, int8_t* qa_h, uint16_t* sa_h, int32_t* asum_h,
                                       bool one_kernel, void* workspace, cudaStream_t stream);
+// the allocation or registration that a byte of host memory lies in; false if the driver knows of none
+bool host_range_of(const void* p, uint64_t* start, uint64_t* size);
 int device_sm_count();                       // SMs of the current device (cached per device)
 int cluster_num_slices(int M, int N, int K);
 // residual: null, or bf16 [M,N] added to the projection before the one rounding (may be y itself)
