@@ -314,10 +314,10 @@ w4a8_status w4a8_linear(const void* x_bf16, const void* packed_w, void* y_bf16,
 /*
  * The whole path for callers whose activations and results live in HOST memory (Sec. 3.5: a
  * pipeline stage is one graph launch fed from the host): enqueues, on `stream`, the copy of
- * x to the device, w4a8_linear, and the copy of y back to the host.  Small requests (512 KiB each way)
- * in pinned memory are not copied: the quantiser reads x in place and, where w4a8_gemm takes the strip or the
- * cluster kernel (w4a8_plan: always up to 16 tokens), y is written in place.  x_dev and y_dev hold x and y afterwards
- * in every case.
+ * x to the device, w4a8_linear, and the copy of y back to the host.  Small requests (512 KiB each way,
+ * K up to 32768) in pinned memory are not copied: the quantiser reads x in place and, where w4a8_gemm takes
+ * the strip or the cluster kernel (w4a8_plan: always up to 16 tokens), y is written in place.  x_dev and y_dev
+ * hold x and y afterwards in every case.
  *   x_host_bf16  HOST [M,K] bf16 (pinned memory makes the copies asynchronous); unchanged until `stream` has passed the call
  *   y_host_bf16  HOST [M,N] bf16, valid once `stream` has been synchronised by the caller
  *   x_dev, qa, sa, asum, y_dev   DEVICE staging buffers owned by the caller, sized and aligned

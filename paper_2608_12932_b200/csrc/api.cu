@@ -75,7 +75,6 @@ bool takes_tcgen05(int M, int N, int K) {
 }
 
 // The device's address of a buffer in pinned host memory, or null if a kernel cannot use it there.
-constexpr size_t HOST_DIRECT_MAX_BYTES = 512 * 1024;
 void* pinned_device_address(const void* p, size_t bytes) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -423,11 +422,8 @@ w4a8_status w4a8_linear_host(const void* x_host_bf16, void* y_host_bf16,
     // microseconds, to move what the kernels themselves move in one or two.  x_dev and y_dev are filled either way.
     const void* x_pinned = nullptr;
     void* y_pinned = nullptr;
-    if ((size_t)M * K * 2 <= HOST_DIRECT_MAX_BYTES) {
-        x_pinned = pinned_device_address(x_host_bf16, (size_t)M * K * 2);
-        if ((size_t)M * N * 2 <= HOST_DIRECT_MAX_BYTES && !takes_tcgen05(M, N, K))
-            y_pinned = pinned_device_address(y_host_bf16, (size_t)M * N * 2);
-    }
+    if (reads_in_place(M, K)) x_pinned = pinned_device_address(x_host_bf16, (size_t)M * K * 2);
+    if (writes_in_place(M, N, K) && !takes_tcgen05(M, N, K)) y_pinned = pinned_device_address(y_host_bf16, (size_t)M * N * 2);
     if (!x_pinned && cudaMemcpyAsync(x_dev, x_host_bf16, (size_t)M * K * 2, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return W4A8_ERR_CUDA;
     w4a8_status s = linear_impl(x_pinned ? x_pinned : x_dev, x_pinned ? x_dev : nullptr, packed_w, y_dev, y_pinned, M, N, K, group,

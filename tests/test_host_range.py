@@ -10,14 +10,21 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 
 
 @pytest.fixture(scope="module")
-def in_place(tmp_path_factory):
+def shim(tmp_path_factory):
     d = tmp_path_factory.mktemp("host_range")
     (d / "shim.cpp").write_text('#include "host_range.h"\n'
                                 'extern "C" uint64_t in_place(int pinned, uint64_t device, uint64_t start, uint64_t size, uint64_t p, uint64_t bytes) {\n'
                                 '    const w4a8::HostMemory m = {pinned != 0, (void*)device, start, size};\n'
-                                '    return (uint64_t)w4a8::in_place_address(m, (const void*)p, bytes);\n}\n')
+                                '    return (uint64_t)w4a8::in_place_address(m, (const void*)p, bytes);\n}\n'
+                                'extern "C" int reads(int M, int K) { return w4a8::reads_in_place(M, K); }\n'
+                                'extern "C" int writes(int M, int N, int K) { return w4a8::writes_in_place(M, N, K); }\n')
     subprocess.run(["g++", "-shared", "-fPIC", "-I", CSRC, "-o", str(d / "shim.so"), str(d / "shim.cpp")], check=True)
-    f = ctypes.CDLL(str(d / "shim.so")).in_place
+    return ctypes.CDLL(str(d / "shim.so"))
+
+
+@pytest.fixture(scope="module")
+def in_place(shim):
+    f = shim.in_place
     f.restype, f.argtypes = ctypes.c_uint64, [ctypes.c_int] + [ctypes.c_uint64] * 5
     return f
 
@@ -39,3 +46,10 @@ def test_what_a_kernel_cannot_address(in_place):
     assert in_place(1, p + 8, p, 4096, p + 8, 64) == 0       # 16-byte accesses would be misaligned
     assert in_place(1, p + 32, p, 0, p, 64) == 0             # no range known
     assert in_place(1, 0x200000, p, 4096, p + 64, 64) == 0x200000      # another address on the device
+
+
+def test_sizes(shim):
+    """Long rows are copied: a CTA that reads one over the bus, twice, is slower than the copy engine."""
+    assert shim.reads(64, 4096) and not shim.reads(65, 4096)
+    assert shim.reads(1, 32768) and shim.reads(8, 32768) and not shim.reads(1, 32896) and not shim.reads(1, 262144)
+    assert shim.writes(8, 32768, 4096) and not shim.writes(9, 32768, 4096) and not shim.writes(1, 128, 65536)
