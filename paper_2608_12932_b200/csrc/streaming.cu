@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(ROPE_WIDE_WARPS * 32)
 rope_shifted_keys_wide_kernel(const uint4* __restrict__ k_pre, const int32_t* __restrict__ pos, int delta, int T, int H, int D,
                               const __grid_constant__ RopeTheta theta, uint4* __restrict__ k_rot) {
     constexpr int U = 2, WARPS = ROPE_WIDE_WARPS;
-    __shared__ float2 rot[WARPS][ROPE_MAX_HALF];             // (cos, sin) of the warp's token
+    __shared__ __align__(16) float2 rot[WARPS][ROPE_MAX_HALF];      // (cos, sin) of the warp's token, read two at a time
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int half = D >> 1, pieces = half >> 3;             // 16-byte pieces per half row
     const int total = H * pieces;                            // ... per token and half

@@ -1,5 +1,5 @@
-"""Source checks of how the kernels wait for one another, which no run can show: a hand-over that a warp acquires through one
-lane is ordered for its other lanes, and no warp waits without a limit for warps that may have given up."""
+"""Source checks of what no run can show: a hand-over that a warp acquires through one lane is ordered for its other lanes, no
+warp waits without a limit for warps that may have given up, and shared memory that is read in 16-byte pieces is declared so."""
 import os
 import re
 
@@ -28,3 +28,12 @@ def test_no_barrier_inside_the_roles_of_the_tensor_core_kernels():
     for name in ("gemm_tcgen05.cu", "gemm_tcshort.cu"):
         text = code(name)
         assert "named_bar_sync" not in text and "bar.sync" not in text and text.count("__syncthreads()") == 2, name
+
+
+def test_shared_tables_read_in_16_byte_pieces_are_aligned():
+    """A float2 table is 8-byte aligned by its type; where the compiler places it today is no promise."""
+    text = code("streaming.cu")
+    names = re.findall(r"reinterpret_cast<const float4\*>\(&(\w+)\[", text)
+    assert names
+    for name in names:
+        assert re.search(r"__shared__ (__align__\(16\) float2|float4) " + name + r"\[", text), name
