@@ -6,17 +6,21 @@
 //   out[i] = k[i] cos(phi) - k[i + D/2] sin(phi),   out[i + D/2] = k[i + D/2] cos(phi) + k[i] sin(phi).
 // One warp per token and all its heads (the angles do not depend on the head).  The angle is formed in fp64, as a number
 // of half turns, and reduced to [-1, 1] there (a position of several thousand times theta_0 = 1 has no bits to spare in
-// fp32); sine and cosine of pi times it are taken in fp32, products and sums in fp32, one rounding to bf16.
+// fp32); sine and cosine of pi times it are taken in fp32, products and sums in fp32, one rounding to bf16.  Both forms
+// below do this with the same numbers in the same order, so that a key's rotation does not depend on which of them a
+// window's size selects.
 // Memory-bound: 2 B in and 2 B out per element.  The wide form takes 16 bytes per lane and half row; a lane's eight
 // neighbouring elements are not the ones whose angles it computed, so a token's sines and cosines go through a small
 // table in shared memory, and theta comes from the host (64 fp64 exponentials in front of a CTA's first load cost a
-// microsecond of latency).  The 4-byte form (any D, any alignment, and few tokens) keeps everything in the lane.
+// microsecond of latency).  The 4-byte form (any D, any alignment, and few tokens) keeps everything in the lane; its theta
+// come from the host too where the wide form could be taken for another window (D <= 2 ROPE_MAX_HALF).
 //
 // streaming_mask_kernel: the new frame's tokens are inserted at the last-frame place of each camera view (the
 // sequence is view-major), only they are queries, and attention stays causal in that order:
 //   mask[q][j] = (j <= position of query q),  position of query (v, i) = ((v F + F - 1) n + i).
 #include <cuda_bf16.h>
 #include <cmath>
+#include <type_traits>
 #include "ptx_sm100.cuh"
 #include "w4a8_internal.cuh"
 
@@ -24,44 +28,69 @@ namespace w4a8 {
 namespace {
 
 constexpr int ROPE_WARPS = 8;
+constexpr int ROPE_MAX_HALF = 128;
+struct RopeTheta { double t[ROPE_MAX_HALF]; };               // theta_i / pi
 
-__global__ void __launch_bounds__(ROPE_WARPS * 32)
+// (cos, sin) of q theta_i
+__device__ __forceinline__ float2 rope_cos_sin(double q, double theta_over_pi) {
+    const double a = __dmul_rn(q, theta_over_pi);
+    float2 cs;
+    sincospif((float)__fma_rn(-2.0, rint(0.5 * a), a), &cs.y, &cs.x);
+    return cs;
+}
+// x, y: two neighbouring elements of the first and of the second half of a row; returns their rotation in place
+__device__ __forceinline__ void rope_rotate2(uint32_t& x, uint32_t& y, float c0, float s0, float c1, float s1) {
+    const float x0 = __uint_as_float(x << 16), x1 = __uint_as_float(x & 0xFFFF0000u);
+    const float y0 = __uint_as_float(y << 16), y1 = __uint_as_float(y & 0xFFFF0000u);
+    x = ptx::pack_bf16x2(fmaf(x0, c0, -__fmul_rn(y0, s0)), fmaf(x1, c1, -__fmul_rn(y1, s1)));
+    y = ptx::pack_bf16x2(fmaf(y0, c0, __fmul_rn(x0, s0)), fmaf(y1, c1, __fmul_rn(x1, s1)));
+}
+
+// TABLE: theta from the host; otherwise (longer half rows) from base ^ (-2 i / D) here.  Eight heads at a time, the rest by
+// code of their own lengths, and four CTAs per SM: with a bounds check per head the compiler keeps 128 to 200 registers of
+// addresses and loads, at half the warps per SM and up to twice the time.  Measured on B200, the angle in radians with checks
+// against this form: 4000 x 8 x 128 5.7 and 4.8 us, 8192 x 4 x 64 6.7 and 5.3, 30000 x 2 x 272 36.2 and 27.0.
+template <bool TABLE>
+__global__ void __launch_bounds__(ROPE_WARPS * 32, 4)
 rope_shifted_keys_kernel(const uint32_t* __restrict__ k_pre, const int32_t* __restrict__ pos, int delta, int T, int H, int D,
-                         double log2_base, uint32_t* __restrict__ k_rot) {
+                         double log2_base, const __grid_constant__ RopeTheta theta, uint32_t* __restrict__ k_rot) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int half = D >> 1, pairs = half >> 1;              // 32-bit words (two bf16) per half row
-    const double two_pi = 6.283185307179586476925286766559, inv_two_pi = 0.15915494309189533576888376337251;
+    __shared__ double th[TABLE ? ROPE_MAX_HALF : 1];         // once per CTA: lanes reading a parameter each at its own index take turns
+    if (TABLE) {
+        for (int i = threadIdx.x; i < half; i += ROPE_WARPS * 32) th[i] = theta.t[i];
+        __syncthreads();
+    }
     for (int w0 = lane; w0 < pairs; w0 += 32) {
         // this lane's elements i = 2 w0 and 2 w0 + 1 of the first half and their partners in the second
-        const double th0 = exp2(-(double)(4 * w0) / (double)D * log2_base), th1 = exp2(-(double)(4 * w0 + 2) / (double)D * log2_base);
+        constexpr double INV_PI = 0.31830988618379067154;
+        const double th0 = TABLE ? th[2 * w0] : exp2(-(double)(4 * w0) / (double)D * log2_base) * INV_PI;
+        const double th1 = TABLE ? th[2 * w0 + 1] : exp2(-(double)(4 * w0 + 2) / (double)D * log2_base) * INV_PI;
         // a warp per token: the angles do not depend on the head, so sine and cosine are taken once for all H rows
         for (int t = blockIdx.x * ROPE_WARPS + warp; t < T; t += gridDim.x * ROPE_WARPS) {
             const double p = (double)(__ldg(pos + t) - delta);
-            double a0 = p * th0, a1 = p * th1;
-            a0 -= two_pi * rint(a0 * inv_two_pi);
-            a1 -= two_pi * rint(a1 * inv_two_pi);
-            float s0, c0, s1, c1;
-            sincosf((float)a0, &s0, &c0);
-            sincosf((float)a1, &s1, &c1);
-            for (int h0 = 0; h0 < H; h0 += 8) {
-                uint32_t lo[8], hi[8];
+            const float2 r0 = rope_cos_sin(p, th0), r1 = rope_cos_sin(p, th1);
+            const uint32_t* src = k_pre + (size_t)t * H * half + w0;
+            uint32_t* dst = k_rot + (size_t)t * H * half + w0;
+            auto heads = [&](auto count) {
+                constexpr int C = decltype(count)::value;
+                uint32_t lo[C], hi[C];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const size_t base_w = ((size_t)t * H + h0 + j) * (D >> 1);
-                    if (h0 + j < H) { lo[j] = __ldg(k_pre + base_w + w0); hi[j] = __ldg(k_pre + base_w + pairs + w0); }
-                }
+                for (int j = 0; j < C; ++j) { lo[j] = __ldg(src + j * half); hi[j] = __ldg(src + j * half + pairs); }
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (h0 + j >= H) break;
-                    const size_t base_w = ((size_t)t * H + h0 + j) * (D >> 1);
-                    const float x0 = __uint_as_float(lo[j] << 16), x1 = __uint_as_float(lo[j] & 0xFFFF0000u);
-                    const float y0 = __uint_as_float(hi[j] << 16), y1 = __uint_as_float(hi[j] & 0xFFFF0000u);
-                    const __nv_bfloat162 olo = __floats2bfloat162_rn(x0 * c0 - y0 * s0, x1 * c1 - y1 * s1);
-                    const __nv_bfloat162 ohi = __floats2bfloat162_rn(y0 * c0 + x0 * s0, y1 * c1 + x1 * s1);
-                    k_rot[base_w + w0] = *reinterpret_cast<const uint32_t*>(&olo);
-                    k_rot[base_w + pairs + w0] = *reinterpret_cast<const uint32_t*>(&ohi);
+                for (int j = 0; j < C; ++j) {
+                    rope_rotate2(lo[j], hi[j], r0.x, r0.y, r1.x, r1.y);
+                    dst[j * half] = lo[j];
+                    dst[j * half + pairs] = hi[j];
                 }
-            }
+                src += C * half;
+                dst += C * half;
+            };
+            int h = 0;
+            for (; h + 8 <= H; h += 8) heads(std::integral_constant<int, 8>());
+            if (H & 4) heads(std::integral_constant<int, 4>());
+            if (H & 2) heads(std::integral_constant<int, 2>());
+            if (H & 1) heads(std::integral_constant<int, 1>());
         }
     }
 }
@@ -69,9 +98,8 @@ rope_shifted_keys_kernel(const uint32_t* __restrict__ k_pre, const int32_t* __re
 // The form for many tokens, half rows of 8 n <= ROPE_MAX_HALF elements and 16-byte-aligned keys: a warp per token, U pairs
 // of 16-byte pieces per lane (first and second half of a row) at a time.  Swept on B200: U = 2 and four warps per CTA, a CTA
 // for every four tokens (persistent warps with the next token's keys requested ahead lose more to their uneven last round).
-constexpr int ROPE_MAX_HALF = 128, ROPE_WIDE_WARPS = 4;
+constexpr int ROPE_WIDE_WARPS = 4;
 constexpr long long ROPE_WIDE_MIN_ELEMENTS = 4 << 20;
-struct RopeTheta { double t[ROPE_MAX_HALF]; };               // theta_i / pi
 __global__ void __launch_bounds__(ROPE_WIDE_WARPS * 32)
 rope_shifted_keys_wide_kernel(const uint4* __restrict__ k_pre, const int32_t* __restrict__ pos, int delta, int T, int H, int D,
                               const __grid_constant__ RopeTheta theta, uint4* __restrict__ k_rot) {
@@ -105,33 +133,21 @@ rope_shifted_keys_wide_kernel(const uint4* __restrict__ k_pre, const int32_t* __
         }
         if (base == 0) {
             const double q = (double)(p - delta);
-            for (int i = lane; i < half; i += 32) {
-                double a = q * th[i];
-                a -= 2.0 * rint(0.5 * a);
-                float2 cs;
-                sincospif((float)a, &cs.y, &cs.x);
-                rot[warp][i] = cs;
-            }
+            for (int i = lane; i < half; i += 32) rot[warp][i] = rope_cos_sin(q, th[i]);
             __syncwarp();
         }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             if (base + lane + 32 * k < total) {
                 const float4* cs = reinterpret_cast<const float4*>(&rot[warp][8 * w[k]]);
-                const uint32_t xs[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w}, ys[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
-                uint32_t ox[4], oy[4];
+                uint32_t xs[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w}, ys[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float4 c = cs[e];                  // cos, sin of element 2 e, then of 2 e + 1
-                    const float x0 = __uint_as_float(xs[e] << 16), x1 = __uint_as_float(xs[e] & 0xFFFF0000u);
-                    const float y0 = __uint_as_float(ys[e] << 16), y1 = __uint_as_float(ys[e] & 0xFFFF0000u);
-                    const __nv_bfloat162 olo = __floats2bfloat162_rn(x0 * c.x - y0 * c.y, x1 * c.z - y1 * c.w);
-                    const __nv_bfloat162 ohi = __floats2bfloat162_rn(y0 * c.x + x0 * c.y, y1 * c.z + x1 * c.w);
-                    ox[e] = *reinterpret_cast<const uint32_t*>(&olo);
-                    oy[e] = *reinterpret_cast<const uint32_t*>(&ohi);
+                    rope_rotate2(xs[e], ys[e], c.x, c.y, c.z, c.w);
                 }
-                k_rot[at[k]] = make_uint4(ox[0], ox[1], ox[2], ox[3]);
-                k_rot[at[k] + pieces] = make_uint4(oy[0], oy[1], oy[2], oy[3]);
+                k_rot[at[k]] = make_uint4(xs[0], xs[1], xs[2], xs[3]);
+                k_rot[at[k] + pieces] = make_uint4(ys[0], ys[1], ys[2], ys[3]);
             }
         }
     }
@@ -153,9 +169,13 @@ streaming_mask_kernel(int V, int F, int n, uint8_t* __restrict__ mask) {
 cudaError_t launch_rope_shifted_keys(const void* k_pre, const int32_t* pos, int delta, int T, int H, int D, double base,
                                      void* k_rot, cudaStream_t stream) {
     int grid = (T + ROPE_WARPS - 1) / ROPE_WARPS;
+    const bool table = D <= 2 * ROPE_MAX_HALF;
+    const double log2_base = log2(base);
+    RopeTheta theta;
+    for (int i = 0; table && i < D / 2; ++i) theta.t[i] = exp2(-(double)(2 * i) / (double)D * log2_base) * 0.31830988618379067154;
     // measured on B200 (cold keys, 4-byte -> wide form): 30000 x 16 x 64 35.8 -> 21.6 us, 16384 x 8 x 128 15.4 -> 13.7, 65536 x 8 x 128
     // 48.5 -> 47.8; 2000 x 8 x 128 3.6 -> 4.4 (one wave of CTAs: the shorter latency chain of the 4-byte form wins)
-    if ((long long)T * H * D >= ROPE_WIDE_MIN_ELEMENTS && D % 16 == 0 && D <= 2 * ROPE_MAX_HALF && ((reinterpret_cast<uintptr_t>(k_pre) | reinterpret_cast<uintptr_t>(k_rot)) & 15) == 0) {
+    if ((long long)T * H * D >= ROPE_WIDE_MIN_ELEMENTS && D % 16 == 0 && table && ((reinterpret_cast<uintptr_t>(k_pre) | reinterpret_cast<uintptr_t>(k_rot)) & 15) == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.stream = stream;
         cudaLaunchAttribute attr;
@@ -163,8 +183,6 @@ cudaError_t launch_rope_shifted_keys(const void* k_pre, const int32_t* pos, int 
         attr.val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        RopeTheta theta;
-        for (int i = 0; i < D / 2; ++i) theta.t[i] = exp2(-(double)(2 * i) / (double)D * log2(base)) * 0.31830988618379067154;
         cfg.gridDim = dim3((unsigned)((T + ROPE_WIDE_WARPS - 1) / ROPE_WIDE_WARPS), 1, 1);
         cfg.blockDim = dim3(ROPE_WIDE_WARPS * 32, 1, 1);
         return cudaLaunchKernelEx(&cfg, rope_shifted_keys_wide_kernel, static_cast<const uint4*>(k_pre), pos, delta, T, H, D, theta,
@@ -172,8 +190,12 @@ cudaError_t launch_rope_shifted_keys(const void* k_pre, const int32_t* pos, int 
     }
     const int cap = device_sm_count() * 8;
     if (grid > cap) grid = cap;
-    rope_shifted_keys_kernel<<<grid, ROPE_WARPS * 32, 0, stream>>>(static_cast<const uint32_t*>(k_pre), pos, delta, T, H, D,
-                                                                   log2(base), static_cast<uint32_t*>(k_rot));
+    if (table)
+        rope_shifted_keys_kernel<true><<<grid, ROPE_WARPS * 32, 0, stream>>>(static_cast<const uint32_t*>(k_pre), pos, delta, T, H, D,
+                                                                             log2_base, theta, static_cast<uint32_t*>(k_rot));
+    else
+        rope_shifted_keys_kernel<false><<<grid, ROPE_WARPS * 32, 0, stream>>>(static_cast<const uint32_t*>(k_pre), pos, delta, T, H, D,
+                                                                              log2_base, theta, static_cast<uint32_t*>(k_rot));
     return cudaGetLastError();
 }
 

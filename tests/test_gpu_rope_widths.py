@@ -33,3 +33,15 @@ def test_widths_and_alignments(T, H, D, offset):
     # half a bf16 step of the exact result (2^-9) widened to the neighbour (2^-8), plus fp32 errors of the two terms
     bound = 2.0 ** -8 * np.abs(ref) + 1e-6 * np.concatenate([terms, terms], axis=2)
     assert np.all(np.abs(onp.bf16_bits_to_f64(out) - ref) <= bound)
+
+
+@pytest.mark.parametrize("T,H,D", [(4096, 8, 128), (5461, 3, 256), (16384, 16, 16)])
+def test_a_key_does_not_depend_on_the_window_around_it(T, H, D):
+    """A window of 4 Mi elements takes the 16-byte form, its parts the 4-byte one: the same bits for the same key."""
+    rng = np.random.default_rng(D)
+    k = t_u16(wl.f32_to_bf16_bits((3.0 * rng.standard_normal((T, H, D))).astype(np.float32)), torch.bfloat16)
+    pos = torch.from_numpy(rng.integers(0, 100000, T).astype(np.int32)).cuda()
+    whole = bits(B.w4a8_rope_shifted_keys(k, pos, 37, 1e6))
+    for lo, hi in ((0, T // 2), (T // 2, T), (17, 18)):
+        part = bits(B.w4a8_rope_shifted_keys(k[lo:hi].contiguous(), pos[lo:hi].contiguous(), 37, 1e6))
+        assert np.array_equal(part, whole[lo:hi])
