@@ -54,7 +54,7 @@ bool small_m_prefers_tcgen05(int M, int N, int K, int sms) {
     const long groups = ((G + S - 1) / S) * ((tiles * S + sms - 1) / sms);
     const long streaming_ns = M <= 32 ? 4200 + 570 * groups : 7000 + 1140 * groups;
     int tile_m = 0, split = 0, balanced = 0;
-    return tcgen05_plan(M, N, K, sms, &tile_m, &split, 4, &balanced) < streaming_ns;      // as the launcher calls it
+    return tcgen05_plan(M, N, K, sms, &tile_m, &split, &balanced) < streaming_ns;      // as the launcher calls it
 }
 
 }  // namespace w4a8
@@ -364,7 +364,7 @@ w4a8_status w4a8_plan(int M, int N, int K, int group, w4a8_plan_info* out) {
     } else {
         p.family = W4A8_PATH_TCGEN05;
         p.strip_rows = 0;
-        tcgen05_plan(M, N, K, sms, &p.tile_m, &p.k_slices, 4, &p.balanced);       // the launcher's own call
+        tcgen05_plan(M, N, K, sms, &p.tile_m, &p.k_slices, &p.balanced);       // the launcher's own call
         const int all = ((M + p.tile_m - 1) / p.tile_m) * tiles;
         p.ctas = p.k_slices > 1 ? all * p.k_slices : (all < sms ? all : sms);
     }

@@ -64,6 +64,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include "dispatch_rules.h"
 #include "ptx_sm100.cuh"
 #include "w4a8_internal.cuh"
 
@@ -872,19 +873,19 @@ cudaError_t launch_per_channel(int tile_m, const int8_t* qa, const uint16_t* sa,
 // 3.6 and 4.2 ns per token and group) and win when there are several waves of them, short ones when a tall tiling would
 // leave SMs idle, and a K split when even the shortest tiling does.  (Against an exhaustive sweep of height, split and
 // walk at 20 to 400 tokens on eight layers the choice is within 6 % of the best.)
-long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max_split, int* balanced) {
+long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* balanced) {
     const int heights[3] = {208, 128, 64};
     const int n_tiles = N / TILE_N, G = K / GROUP;
     long best_ns = -1;
     *tile_m = 64;
     *split = 1;
-    if (balanced) *balanced = 0;
+    *balanced = 0;
     for (int i = 0; i < 3; ++i) {
         if (heights[i] > 64 && M <= heights[i + 1]) continue;        // the next height down already covers M in one tile
         const long tiles = (long)((M + heights[i] - 1) / heights[i]) * n_tiles;
         const long waves = (tiles + sms - 1) / sms;
         const long group_ns = M <= 32 ? TC_GROUP_32_NS : TC_GROUP_NS[i];
-        for (int S = 1; S <= TC_MAX_SPLIT && S <= max_split; ++S) {
+        for (int S = 1; S <= TC_MAX_SPLIT; ++S) {
             if (S > 1) {
                 if (tiles * S > sms || G / S < 4) break;
                 const int room = i == 0 ? max_active_clusters<208>(S) : (i == 1 ? max_active_clusters<128>(S) : max_active_clusters<64>(S));
@@ -893,11 +894,11 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max
             const long ns = TC_FIXED_NS[i] + waves * group_ns * ((G + S - 1) / S) + TC_SPLIT_NS[i][S];
             if (best_ns < 0 || ns < best_ns) {                        // ties: taller tile, fewer slices
                 best_ns = ns; *tile_m = heights[i]; *split = S;
-                if (balanced) *balanced = 0;
+                *balanced = 0;
             }
             // no split, more tiles than SMs: an even share of all tiles x groups units per CTA, at the price of
             // handing partial tiles over between neighbours
-            if (S == 1 && balanced && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
+            if (S == 1 && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
                 const long nb = TC_FIXED_NS[i] + group_ns * ((tiles * G + sms - 1) / sms) * TC_BALANCE_PERCENT[i] / 100 + TC_BALANCE_NS[i];
                 if (nb < best_ns) { best_ns = nb; *tile_m = heights[i]; *split = 1; *balanced = 1; }
             }
@@ -910,7 +911,7 @@ cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const int3
                                 int M, int N, int K, void* workspace, int32_t* debug_partials,
                                 cudaStream_t stream) {
     int tile_m = 64, S = 1, balanced = 0;
-    tcgen05_plan(M, N, K, device_sm_count(), &tile_m, &S, TC_MAX_SPLIT, &balanced);
+    tcgen05_plan(M, N, K, device_sm_count(), &tile_m, &S, &balanced);
     if (residual)                                   // (no partials dump in this form)
         return launch_plan<false, true>(tile_m, S, balanced != 0, qa, sa, asum, packed, y, residual, M, N, K, workspace, nullptr, stream);
     if (debug_partials)
@@ -923,8 +924,7 @@ cudaError_t launch_gemm_tcgen05(const int8_t* qa, const uint16_t* sa, const int3
 cudaError_t launch_gemm_tcgen05_per_channel(const int8_t* qa, const uint16_t* sa, const void* packed, void* y,
                                             int M, int N, int K, void* workspace, int32_t* debug_sums,
                                             cudaStream_t stream) {
-    int tile_m = 64, S = 1;
-    tcgen05_plan(M, N, K, device_sm_count(), &tile_m, &S, 1, nullptr);
+    const int tile_m = per_channel_tile_height(M, N / TILE_N, K / GROUP, device_sm_count());
     if (debug_sums)
         return launch_per_channel<true>(tile_m, qa, sa, packed, y, M, N, K, workspace, debug_sums, stream);
     return launch_per_channel<false>(tile_m, qa, sa, packed, y, M, N, K, workspace, nullptr, stream);

@@ -132,9 +132,8 @@ cudaError_t launch_gemm_tcshort(int S, bool balanced, const int8_t* qa, const ui
                                 const void* packed, void* y, const void* residual, int M, int N, int K, void* workspace,
                                 int32_t* debug_partials, cudaStream_t stream);
 int tcshort_max_clusters(int S);
-// tile height, K split (at most max_split slices) and, if asked for, whether the balanced walk is taken, as the
-// tcgen05 launcher picks them; returns its time estimate (ns)
-long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int max_split = 4, int* balanced = nullptr);
+// tile height, K split and whether the balanced walk is taken, as the launcher picks them for the grouped form; returns its time estimate (ns)
+long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* balanced);
 bool small_m_prefers_tcgen05(int M, int N, int K, int sms);
 
 }  // namespace w4a8
