@@ -26,4 +26,19 @@ inline int per_channel_tile_height(int M, int n_tiles, int groups, int sms) {
     return best;
 }
 
+// CTAs that share a row in the SiLU quantiser (a cluster; 1: one CTA per row), by rows and channels: a cluster's start and two
+// barriers pay only where a row is long and the rows are few.  Measured on B200 on both sides of each line, time with the
+// cluster over time with one CTA per row, alone and behind two sizes of the projection: 16 rows of 4096 channels 1.05 (alone),
+// of 5120 0.84 to 0.94; 24 of 6144 0.89, 1.23 and 1.17, of 8192 0.84 to 0.99; 48 of 4096 0.99 to 1.06, of 5120 0.82 to 0.93; 64 of
+// 5120 1.06 to 1.10, of 8192 0.89 to 1.00; 96 of 8192 0.98 to 1.01, of 12288 0.91 to 0.97; 160 of 6144 0.93 to 1.03, of 8192 0.80 to
+// 0.99; 200 of 6144 1.18 alone and 0.95 to 0.98 behind, of 8192 1.02 and 0.89 to 0.92; 300 of 6144 0.99 to 1.09, of 10240 0.89
+// to 0.97; 700 of 10240 1.03 to 1.11.  On short rows it is up to twice as long (256 of 512 alone: 4.9 and 2.5 us).
+inline int silu_cluster_ctas(int M, int K) {
+    struct Line { int rows, min_channels, ctas; };
+    constexpr Line LINES[] = {{16, 5120, 8}, {32, 8192, 8}, {48, 5120, 8}, {64, 8192, 8}, {128, 12288, 8}, {160, 8192, 8}, {256, 8192, 4}, {600, 10240, 2}};
+    for (const Line& l : LINES)
+        if (M <= l.rows) return K >= l.min_channels ? l.ctas : 1;
+    return 1;
+}
+
 }  // namespace w4a8

@@ -12,6 +12,7 @@
 // division.  Eight instructions per element instead of about thirty.  Group sums of the codes (the
 // zero-point correction term) come from a 16-lane segmented shuffle: 16 chunks of 8 = one group of 128.
 #include <cuda_fp16.h>
+#include "dispatch_rules.h"
 #include "ptx_sm100.cuh"
 #include "quant_common.cuh"
 #include "w4a8_internal.cuh"
@@ -162,7 +163,7 @@ quantize_act_kernel(const uint4* __restrict__ x, int K, uint2* __restrict__ qa,
 // The SiLU form for few rows: a row of the fused gate+up projection is shared by a cluster of C CTAs of T threads, R
 // chunks per thread kept in registers.  Each CTA forms h and finds the maximum over its share of the groups, tells it to
 // the others through distributed shared memory, and quantises its share.  With one CTA per row the kernel above is a
-// latency chain on a few SMs (12288 channels: 5.1 us at 40 rows, 10.0 at 150); shared, 4.4 and 6.3 us.
+// latency chain on a few SMs (12288 channels alone: 4.5 us at 8 rows, 5.6 at 64, 10.4 at 160; shared, 2.7, 4.3 and 6.9).
 template <int T, int R>
 __global__ void __launch_bounds__(T)
 silu_quantize_cluster_kernel(const uint4* __restrict__ x, int K, int C, uint2* __restrict__ qa, uint16_t* __restrict__ sa,
@@ -274,10 +275,10 @@ cudaError_t launch_quantize(const void* x, int M, int K, int8_t* qa, uint16_t* s
     const uint4* xp = reinterpret_cast<const uint4*>(x);
     uint2* qp = reinterpret_cast<uint2*>(qa);
     uint4* hp = reinterpret_cast<uint4*>(h_out);
-    if (SILU && M <= 700) {
-        // measured on B200 at 12288 channels, one CTA per row -> cluster: 20 rows 4.7 -> 2.9 us, 64 5.5 -> 4.3, 200 7.6 ->
-        // 6.9, 300 10.7 -> 9.1, 512 14.3 -> 12.7; 1024 rows and more are equal or slower (the machine is full either way)
-        const int C = M <= 160 ? 8 : (M <= 256 ? 4 : 2), T = M > 32 && M <= 160 ? 128 : 256;
+    const int C = SILU ? silu_cluster_ctas(M, K) : 1;
+    if (C > 1) {
+        // (a share of more than 256 chunks at 33 to 160 rows, or of more than 1024: one CTA per row, below)
+        const int T = M > 32 && M <= 160 ? 128 : 256;
         const int own = (K / GROUP + C - 1) / C * 16, R = (own + T - 1) / T;
         if (T == 128) {
             if (R == 1) return launch_silu_cluster<128, 1>(cfg, M, C, xp, K, qp, sa, asum, hp);

@@ -14,7 +14,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("M,I", [(1, 128), (17, 384), (32, 13824), (33, 1152), (160, 6144), (161, 6144), (256, 2176), (257, 12288),
-                                 (700, 1280), (701, 1280), (40, 25600)])
+                                 (700, 1280), (701, 1280), (40, 25600), (1, 5120), (16, 5248), (17, 8192), (32, 28672), (33, 5120),
+                                 (48, 13824), (49, 8320), (65, 12288), (128, 12416), (129, 8192), (160, 16384), (160, 16512), (161, 8192),
+                                 (256, 10368), (257, 10240), (600, 10240), (601, 10240)])
 def test_rows_and_channel_shares(M, I):
     rng = np.random.default_rng(M + I)
     y = wl.f32_to_bf16_bits((rng.standard_normal((M, 2 * I)) * 2).astype(np.float32))
