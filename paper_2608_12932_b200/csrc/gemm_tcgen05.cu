@@ -79,11 +79,17 @@ constexpr int RAW_STRIDE = 8576;                 // BLOB_BYTES rounded up to a m
 constexpr int A_COLS = GROUP / 4;                // 32 TMEM columns hold one group of a weight row (4 bytes per column)
 constexpr int TMEM_COLS = 512;
 // Cost model of tcgen05_plan (nanoseconds, measured on B200 behind the quantiser, weights cold; 208-, 128-, 64-row
-// tiles): per launch; per group a CTA walks; for splitting K over a cluster of S CTAs (two cluster barriers, exchange and
-// reduction); for the balanced walk (hand-over of two partial tiles, and CTAs out of step: its groups in per cent of the plain walk's).  64-row tiles run
-// in the kernel of gemm_tcshort.cu, whose tile is cut to 32 columns for up to 32 tokens.
+// tiles): per launch; per group a CTA walks; per tile after a CTA's first (its epilogue); for splitting K over a cluster of S
+// CTAs (two cluster barriers, exchange and reduction); for the balanced walk (hand-over of two partial tiles, and CTAs out of
+// step: its groups in per cent of the plain walk's).  64-row tiles run in the kernel of gemm_tcshort.cu, whose tile is cut to
+// 32 columns for up to 32 tokens.
+// A tile of few groups is mostly epilogue, so layers of up to 15 groups have constants of their own: fitted to every height
+// at 14 token counts from 65 on and six widths, the choice is within 3 % of the best height (with the constants for long K up to
+// 16 %: 768 -> 24576 at 96 tokens 11.9 us with 64 rows and 10.8 with 128).  From 16 groups on the epilogue is in the fit of the others.
 constexpr int TC_MAX_SPLIT = 4;
-constexpr long TC_FIXED_NS[3] = {3500, 3200, 2500}, TC_GROUP_NS[3] = {525, 440, 255}, TC_GROUP_32_NS = 230;
+struct TcCost { long fixed[3], group[3], tile[3]; };
+constexpr TcCost TC_COST = {{3500, 3200, 2500}, {525, 440, 255}, {0, 0, 0}}, TC_COST_MEDIUM = {{4000, 2550, 2500}, {525, 440, 255}, {2350, 1450, 1250}};
+constexpr long TC_GROUP_32_NS = 230;
 constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 4000, 4500, 5600}, {0, 0, 2800, 2800, 3400}, {0, 0, 1800, 2700, 3500}};
 constexpr long TC_BALANCE_NS[3] = {6000, 4000, 4500}, TC_BALANCE_PERCENT[3] = {104, 104, 100};
 
@@ -868,14 +874,15 @@ cudaError_t launch_per_channel(int tile_m, const int8_t* qa, const uint16_t* sa,
 }  // namespace
 
 // Tile height and K split for an [M, N, K] problem, from a cost model fitted to measurements on B200: a CTA spends
-// about TC_FIXED_NS on launch, set-up and pipeline fill, then TC_GROUP_NS[height] per 128-k group of every tile it
-// walks; a K split into S slices costs TC_SPLIT_NS for the cluster exchange.  Tall tiles are cheapest per token (2.6,
+// a fixed time on launch, set-up and pipeline fill, then one per 128-k group of every tile it walks, by height (TC_COST);
+// a K split into S slices costs TC_SPLIT_NS for the cluster exchange.  Tall tiles are cheapest per token (2.6,
 // 3.6 and 4.2 ns per token and group) and win when there are several waves of them, short ones when a tall tiling would
 // leave SMs idle, and a K split when even the shortest tiling does.  (Against an exhaustive sweep of height, split and
 // walk at 20 to 400 tokens on eight layers the choice is within 6 % of the best.)
 long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* balanced) {
     const int heights[3] = {208, 128, 64};
     const int n_tiles = N / TILE_N, G = K / GROUP;
+    const TcCost& cost = M > 32 && G < 16 ? TC_COST_MEDIUM : TC_COST;
     long best_ns = -1;
     *tile_m = 64;
     *split = 1;
@@ -884,14 +891,15 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* ba
         if (heights[i] > 64 && M <= heights[i + 1]) continue;        // the next height down already covers M in one tile
         const long tiles = (long)((M + heights[i] - 1) / heights[i]) * n_tiles;
         const long waves = (tiles + sms - 1) / sms;
-        const long group_ns = M <= 32 ? TC_GROUP_32_NS : TC_GROUP_NS[i];
+        const long group_ns = M <= 32 ? TC_GROUP_32_NS : cost.group[i];
+        const long fixed_ns = cost.fixed[i] + (waves - 1) * cost.tile[i];
         for (int S = 1; S <= TC_MAX_SPLIT; ++S) {
             if (S > 1) {
                 if (tiles * S > sms || G / S < 4) break;
                 const int room = i == 0 ? max_active_clusters<208>(S) : (i == 1 ? max_active_clusters<128>(S) : max_active_clusters<64>(S));
                 if (tiles > room) continue;                          // the clusters must all be resident at once
             }
-            const long ns = TC_FIXED_NS[i] + waves * group_ns * ((G + S - 1) / S) + TC_SPLIT_NS[i][S];
+            const long ns = fixed_ns + waves * group_ns * ((G + S - 1) / S) + TC_SPLIT_NS[i][S];
             if (best_ns < 0 || ns < best_ns) {                        // ties: taller tile, fewer slices
                 best_ns = ns; *tile_m = heights[i]; *split = S;
                 *balanced = 0;
@@ -899,7 +907,7 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* ba
             // no split, more tiles than SMs: an even share of all tiles x groups units per CTA, at the price of
             // handing partial tiles over between neighbours
             if (S == 1 && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
-                const long nb = TC_FIXED_NS[i] + group_ns * ((tiles * G + sms - 1) / sms) * TC_BALANCE_PERCENT[i] / 100 + TC_BALANCE_NS[i];
+                const long nb = fixed_ns + group_ns * ((tiles * G + sms - 1) / sms) * TC_BALANCE_PERCENT[i] / 100 + TC_BALANCE_NS[i];
                 if (nb < best_ns) { best_ns = nb; *tile_m = heights[i]; *split = 1; *balanced = 1; }
             }
         }

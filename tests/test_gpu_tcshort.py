@@ -49,7 +49,7 @@ def test_uneven_k_split(M, K, N):
     assert np.array_equal(y, check(case, layer, M, debug=False))
 
 
-@pytest.mark.parametrize("M,K,N", [(20, 1152, 24576), (40, 1152, 24576), (300, 1152, 4352)])
+@pytest.mark.parametrize("M,K,N", [(20, 1152, 24576), (40, 1152, 24576), (130, 1152, 24576)])
 def test_more_tiles_than_sms(M, K, N):
     """More tiles than SMs, nine groups each, as whole tiles: rings and accumulator buffers run on from one tile to the next
     behind a lone last group.  (Tiles shared by neighbouring CTAs: test_gpu_balanced_walk.py.)"""

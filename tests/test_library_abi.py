@@ -175,3 +175,10 @@ def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     monkeypatch.setattr(B, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no fallback"):
         B.lib()
+
+
+def test_tile_height_of_layers_with_few_groups():
+    """A tile of few groups is mostly epilogue: taller tiles in fewer rounds, as measured with every height forced."""
+    for M, N, K, tile in ((200, 8192, 1024, 128), (256, 8192, 768, 128), (96, 24576, 1024, 128), (400, 4096, 1024, 128), (700, 8192, 1024, 208),
+                          (400, 24576, 1024, 208), (100, 8192, 1024, 64), (64, 24576, 1024, 64)):
+        assert B.w4a8_plan(M, N, K)["tile_m"] == tile, (M, N, K)
