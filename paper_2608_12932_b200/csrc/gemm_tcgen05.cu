@@ -1,5 +1,5 @@
 // Large-M W4A8 GEMM for sm_100a (token tiles of 208 and 128 rows; 64-row tiles, for fewer tokens, run in
-// gemm_tcshort.cu - only the per-channel form below has them here): bulk copies -> shared memory -> int4->int8 unpack into TENSOR
+// gemm_tcshort.cu - the per-channel form below has them here, and layers of up to four groups at more than 32 tokens): bulk copies -> shared memory -> int4->int8 unpack into TENSOR
 // MEMORY -> tcgen05.mma kind::i8 (weights from TMEM, activations from shared memory) with int32
 // accumulators in TMEM -> per-group fp32 scaling -> bf16.
 // (Sec. 3.4: quantising the activations to 8 bits is what lets the compute-bound prefill run on
@@ -85,10 +85,17 @@ constexpr int TMEM_COLS = 512;
 // 32 columns for up to 32 tokens.
 // A tile of few groups is mostly epilogue, so layers of up to 15 groups have constants of their own: fitted to every height
 // at 14 token counts from 65 on and six widths, the choice is within 3 % of the best height (with the constants for long K up to
-// 16 %: 768 -> 24576 at 96 tokens 11.9 us with 64 rows and 10.8 with 128).  From 16 groups on the epilogue is in the fit of the others.
+// 16 %: 768 -> 24576 at 96 tokens 11.9 us with 64 rows and 10.8 with 128), up to four groups within 11 %.  From 16 groups on the epilogue is in the fit of the others.
 constexpr int TC_MAX_SPLIT = 4;
 struct TcCost { long fixed[3], group[3], tile[3]; };
-constexpr TcCost TC_COST = {{3500, 3200, 2500}, {525, 440, 255}, {0, 0, 0}}, TC_COST_MEDIUM = {{4000, 2550, 2500}, {525, 440, 255}, {2350, 1450, 1250}};
+constexpr TcCost TC_COST = {{3500, 3200, 2500}, {525, 440, 255}, {0, 0, 0}}, TC_COST_MEDIUM = {{4000, 2550, 2500}, {525, 440, 255}, {2350, 1450, 1250}},
+                 TC_COST_FEW = {{4550, 3750, 2950}, {800, 605, 405}, {2400, 1500, 1250}};
+// Layers of up to four groups at more than 32 tokens run their 64-row tiles here: the kernel of gemm_tcshort.cu gains 0.15 us a
+// group and loses 0.4 to 0.5 before its first and after its last (measured on B200 behind the quantiser, here against there: 128
+// -> 8192 at 64 tokens 4.5 and 5.0 us, 384 -> 24576 at 64 6.5 and 7.3, 512 -> 1024 at 128 5.1 and 5.5; 768 -> 1024 equal, 1024 -> 24576
+// at 64 10.1 and 9.7; up to 32 tokens, where its tile has 32 columns, 256 -> 24576 5.9 and 5.7).
+constexpr int TC_FEW_GROUPS = 4;
+bool few_groups(int M, int G) { return M > 32 && G <= TC_FEW_GROUPS; }
 constexpr long TC_GROUP_32_NS = 230;
 constexpr long TC_SPLIT_NS[3][TC_MAX_SPLIT + 1] = {{0, 0, 4000, 4500, 5600}, {0, 0, 2800, 2800, 3400}, {0, 0, 1800, 2700, 3500}};
 constexpr long TC_BALANCE_NS[3] = {6000, 4000, 4500}, TC_BALANCE_PERCENT[3] = {104, 104, 100};
@@ -849,6 +856,8 @@ int max_active_clusters(int S) {
 template <bool DEBUG, bool RES = false>
 cudaError_t launch_plan(int tile_m, int S, bool balanced, const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
                         const void* residual, int M, int N, int K, void* workspace, int32_t* debug_partials, cudaStream_t stream) {
+    if (tile_m == 64 && few_groups(M, K / GROUP))       // (neither split nor balanced: the planner does neither with so few groups)
+        return launch_tile<64, DEBUG, false, false, false, RES>(qa, sa, packed, y, residual, M, N, K, 1, workspace, debug_partials, stream);
     if (tile_m == 64)
         return launch_gemm_tcshort(S, balanced, qa, sa, asum, packed, y, residual, M, N, K, workspace, debug_partials, stream);
     if (S > 1) {
@@ -882,7 +891,7 @@ cudaError_t launch_per_channel(int tile_m, const int8_t* qa, const uint16_t* sa,
 long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* balanced) {
     const int heights[3] = {208, 128, 64};
     const int n_tiles = N / TILE_N, G = K / GROUP;
-    const TcCost& cost = M > 32 && G < 16 ? TC_COST_MEDIUM : TC_COST;
+    const TcCost& cost = few_groups(M, G) ? TC_COST_FEW : (M > 32 && G < 16 ? TC_COST_MEDIUM : TC_COST);
     long best_ns = -1;
     *tile_m = 64;
     *split = 1;
@@ -906,7 +915,7 @@ long tcgen05_plan(int M, int N, int K, int sms, int* tile_m, int* split, int* ba
             }
             // no split, more tiles than SMs: an even share of all tiles x groups units per CTA, at the price of
             // handing partial tiles over between neighbours
-            if (S == 1 && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
+            if (S == 1 && G > TC_FEW_GROUPS && tiles > sms && tiles % sms != 0 && sms <= HANDOVER_SLOTS && handover_bytes(M, N, K) > 0) {
                 const long nb = fixed_ns + group_ns * ((tiles * G + sms - 1) / sms) * TC_BALANCE_PERCENT[i] / 100 + TC_BALANCE_NS[i];
                 if (nb < best_ns) { best_ns = nb; *tile_m = heights[i]; *split = 1; *balanced = 1; }
             }

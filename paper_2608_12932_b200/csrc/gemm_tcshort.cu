@@ -1,4 +1,5 @@
-// W4A8 GEMM on the tensor cores for token tiles of 64 rows (17 to a few hundred tokens): the scheme of
+// W4A8 GEMM on the tensor cores for token tiles of 64 rows (17 to a few hundred tokens, layers of more than four groups;
+// up to 32 tokens any layer): the scheme of
 // gemm_tcgen05.cu - weights as bytes in tensor memory, tokens on the MMA's N side, one drain per quantisation group.
 // (Sec. 3.4: INT8 tensor cores; Sec. 4: between decode and prefill a call is bound by neither alone.)
 //

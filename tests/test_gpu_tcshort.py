@@ -25,9 +25,10 @@ def check(case, layer, M, debug=True):
     return y
 
 
-@pytest.mark.parametrize("K,N", [(128, 128), (256, 256), (384, 128), (640, 384), (1664, 256), (2304, 384)])
+@pytest.mark.parametrize("K,N", [(128, 128), (256, 256), (384, 128), (512, 256), (640, 384), (1664, 256), (2304, 384)])
 def test_group_counts_and_tile_edges(K, N):
-    """1, 2, 3, 5, 13 and 18 groups; token counts at the edges of the 16-column MMA steps, of both tiles and of several tiles."""
+    """1, 2, 3, 4, 5, 13 and 18 groups; token counts at the edges of the 16-column MMA steps, of both tiles and of several tiles.  (Up
+    to four groups, more than 32 tokens take the 64-row tiles of gemm_tcgen05.cu: their first and last sizes are here too.)"""
     case = wl.make_layer(K, N, 60 + K // 128, 130)
     layer = DeviceLayer(case, 130)
     for M in (1, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129):
@@ -61,11 +62,11 @@ def test_more_tiles_than_sms(M, K, N):
     assert np.array_equal(y1, check(case, layer, M, debug=False))
 
 
-@pytest.mark.parametrize("M", [17, 64])
-def test_extreme_partials(M):
+@pytest.mark.parametrize("M,K", [(17, 384), (64, 384), (33, 640), (64, 640)])
+def test_extreme_partials(M, K):
     """Codes and zero points at the ends of their ranges against activation codes at +-127: |D| = 243840, the bias is 245760."""
     rng = np.random.default_rng(5)
-    K, N = 384, 256
+    N = 256
     case = wl.random_codes(rng, M, N, K)
     case["qw"][:] = np.where(rng.integers(0, 2, (N, 1)) == 1, 15, 0)
     case["z"][:] = np.where(case["qw"][:, 0] == 15, 0, 15)[None, :]

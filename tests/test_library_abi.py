@@ -180,5 +180,6 @@ def test_missing_library_fails_loudly(tmp_path, monkeypatch):
 def test_tile_height_of_layers_with_few_groups():
     """A tile of few groups is mostly epilogue: taller tiles in fewer rounds, as measured with every height forced."""
     for M, N, K, tile in ((200, 8192, 1024, 128), (256, 8192, 768, 128), (96, 24576, 1024, 128), (400, 4096, 1024, 128), (700, 8192, 1024, 208),
-                          (400, 24576, 1024, 208), (100, 8192, 1024, 64), (64, 24576, 1024, 64)):
+                          (400, 24576, 1024, 208), (100, 8192, 1024, 64), (64, 24576, 1024, 64), (512, 8192, 512, 128), (700, 8192, 512, 208), (1024, 24576, 256, 208),
+                          (300, 24576, 384, 128), (128, 1024, 512, 64)):
         assert B.w4a8_plan(M, N, K)["tile_m"] == tile, (M, N, K)
