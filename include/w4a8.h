@@ -205,7 +205,7 @@ w4a8_status w4a8_gemm_residual(w4a8_path path, const int8_t* qa, const uint16_t*
  *                            become visible costs more than a dependent launch), kept for comparison.
  *   W4A8_GATE_UP_SEPARATE    w4a8_gemm into y_scratch, then w4a8_silu_mul_quantize.  Any M.
  *   W4A8_GATE_UP_AUTO        EPILOGUE where w4a8_gemm would take the strip kernel, else SEPARATE (w4a8_gate_up_form says
- *                            which, 0 for an unsupported shape).
+ *                            which, 0 for an unsupported shape); EPILOGUE as well where y_scratch is NULL and M <= 16.
  *   qa, sa, asum, packed_gate_up, M, N (= 2 I), K, group, workspace: as for w4a8_gemm
  *   h          device, bf16 [M, I]: output, and in the first two forms also the buffer through which h reaches the
  *              warps that quantise it (required)

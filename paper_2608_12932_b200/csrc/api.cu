@@ -61,13 +61,20 @@ bool small_m_prefers_tcgen05(int M, int N, int K, int sms) {
 
 namespace {
 
-// Where w4a8_gemm takes the strip kernel: up to 8 tokens always; from 9 to 16 tokens (two token blocks per warp) unless a
-// long K meets so few strips that splitting K over a cluster pays.  Measured on B200 at 16 tokens, strip against cluster
-// kernel: 2048 -> 2048 3.1 and 6.7 us, 4096 -> 4096 5.0 and 5.6, 12288 -> 4096 9.6 and 9.8, 13824 -> 5120 12.5 and 17.7,
-// 2048 -> 1024 3.1 and 3.4; but 8192 -> 1024 5.9 and 5.0, 16384 -> 128 9.6 and 6.5.
+// Where w4a8_gemm takes the strip kernel: up to 8 tokens always; from 9 to 16 tokens (two token blocks per warp) unless
+//  * a long K meets so few strips that splitting K over a cluster pays.  Measured on B200 at 16 tokens behind the quantiser,
+//    strip against cluster kernel: 2048 -> 1024 4.8 and 5.1 us, 4096 -> 1024 6.3 and 5.9, 8192 -> 1024 9.0 and 7.4, 16384 -> 128 13.8
+//    and 10.6; 2048 -> 2048 4.8 and 8.2, 8192 -> 2048 8.6 and 12.3, 28672 -> 2048 24.7 and 27.3, 12288 -> 4096 12.0 and 12.4, 28672 ->
+//    4096 26.2 and 25.5, 12288 -> 5120 14.8 and 19.3;
+//  * a short K meets many strips, each of which then costs its sums and its store and streams little: 128 -> 1024 4.2 and 4.1,
+//    128 -> 24576 11.0 and 4.7, 512 -> 5120 5.6 and 5.1, 512 -> 24576 10.7 and 6.7, 1024 -> 12288 6.8 and 6.1, 1536 -> 24576 12.8 and
+//    11.2; but 256 -> 4096 4.6 and 4.7, 768 -> 5120 5.3 and 5.5, 1024 -> 8192 5.2 and 5.8, 2048 -> 12288 9.0 and 8.6, 2048 -> 24576 13.1
+//    and 13.3.
 bool auto_takes_strip(int M, int N, int K) {
     if (!strip_supported(M, N, K)) return false;
-    return M <= 8 || N >= 2048 || K <= 2048;
+    if (M <= 8) return true;
+    if ((K <= 128 && N >= 1024) || (K <= 512 && N >= 5120) || (K <= 1536 && N >= 12288)) return false;
+    return N >= 2048 || K <= 2048;
 }
 
 bool takes_tcgen05(int M, int N, int K) {
@@ -258,7 +265,11 @@ w4a8_status w4a8_gate_up_silu_quantize(int form, const int8_t* qa, const uint16_
         form != W4A8_GATE_UP_SEPARATE)
         return W4A8_ERR_SHAPE;
     if (M == 0) return W4A8_OK;
-    if (form == W4A8_GATE_UP_AUTO) form = w4a8_gate_up_form(M, N, K, group);
+    if (form == W4A8_GATE_UP_AUTO) {
+        form = w4a8_gate_up_form(M, N, K, group);
+        // without a scratch the epilogue form, wherever it exists
+        if (form == W4A8_GATE_UP_SEPARATE && !y_scratch_bf16 && strip_supported(M, N, K)) form = W4A8_GATE_UP_EPILOGUE;
+    }
     // the two forms that live in the strip kernel's epilogue exist where that kernel does
     if (form != W4A8_GATE_UP_SEPARATE && !strip_supported(M, N, K)) return W4A8_ERR_SHAPE;
     if (!qa || !sa || !asum || !packed_gate_up || !h_bf16 || !qa_h || !sa_h || !asum_h || !workspace) return W4A8_ERR_NULL;

@@ -73,14 +73,14 @@ constexpr int ST_EPILOGUE_WARP = ST_CONSUMER_WARPS + ST_PRODUCER_WARPS;
 constexpr int ST_THREADS = (ST_CONSUMER_WARPS + ST_PRODUCER_WARPS + 1) * 32;
 constexpr int ST_MAX_STAGES = 8;
 constexpr int ST_W_BYTES = ST_CW == 8 ? 17408 : (ST_CW == 12 ? 26624 : 34816);                         // weight part of a stage (16 KB of nibbles + scales + zero points, padded)
-// CTAs per SM.  Up to 8 tokens two: the second CTA's warps multiply while the first one's wait for data.  With two token
-// blocks one, with twice the ring and up to 168 registers a thread: at 80 the second block's fragments and sums leave no
-// room for the loads of the next unit, and every stage waits for its shared-memory round trips in turn (4096 -> 24576 at 16
-// tokens 19.2 us with two, 17.1 with one; 5120 -> 27648 26.3 and 23.4; 12288 -> 4096 with residual 16.9 and 9.6; the other
-// way round up to 8 tokens: 4096 -> 24576 12.9 and 14.7).  Twelve or sixteen consumer warps in one CTA per SM are 2 to 20 %
-// slower on most layers.
-__host__ __device__ constexpr int st_ctas_per_sm(int mb) { return mb == 1 ? 2 : 1; }
-__host__ __device__ constexpr int st_smem_budget(int mb) { return (mb == 1 ? 112 : 220) * 1024; }
+// CTAs per SM (the template's CTAS).  Up to 8 tokens two: the second CTA's warps multiply while the first one's wait for data.
+// With two token blocks one, with twice the ring and up to 168 registers a thread: at 80 the second block's fragments and sums
+// leave no room for the loads of the next unit, and every stage waits for its shared-memory round trips in turn (4096 ->
+// 24576 at 16 tokens 19.2 us with two, 17.1 with one; 5120 -> 27648 26.3 and 23.4; 12288 -> 4096 with residual 16.9 and 9.6;
+// the other way round up to 8 tokens: 4096 -> 24576 12.9 and 14.7) - but for a short K of few more strips than SMs, where one
+// CTA per SM means shared strips and two do not (strip_plan).  Twelve or sixteen consumer warps in one CTA per SM are 2 to
+// 20 % slower on most layers.
+__host__ __device__ constexpr int st_smem_budget(int ctas_per_sm) { return (ctas_per_sm == 2 ? 112 : 220) * 1024; }
 constexpr uint32_t ST_STAY = 128;                         // one-kernel fused form: CTAs that stay to requantise (swept 32..296 on B200)
 constexpr int ST_MAX_ASUM_WORDS = 4096;                   // group sums of all tokens kept in shared memory
 
@@ -209,8 +209,8 @@ struct StripArgs {
 // counts itself in; the last 128 to do so stay, wait (bounded) until the count is complete, and quantise.
 // FUSE == 3 is unrelated to gate+up: the plain projection with a residual added at the store (fp32 staging, the
 // residual's 16-byte pieces requested before the wait for the consumers), for the O and down projections.
-template <int MB, int RBLK, bool DEBUG, int FUSE>
-__global__ void __launch_bounds__(ST_THREADS, st_ctas_per_sm(MB))
+template <int MB, int RBLK, bool DEBUG, int FUSE, int CTAS>
+__global__ void __launch_bounds__(ST_THREADS, CTAS)
 gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_constant__ CUtensorMap tm_nib,
                   const __grid_constant__ CUtensorMap tm_scale, const __grid_constant__ CUtensorMap tm_zero,
                   const StripArgs a) {
@@ -800,7 +800,7 @@ struct FuseOut {
     bool one_kernel;
 };
 
-template <int MB, int RBLK, bool DEBUG, int FUSE>
+template <int MB, int RBLK, bool DEBUG, int FUSE, int CTAS>
 cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
                          const void* residual, void* y_copy, int M, int N, int K, int ctas, void* workspace,
                          int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
@@ -808,7 +808,7 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     const int G = K / GROUP;
     const bool fp32_stage = FUSE == 3;
     const int fixed = st_layout(MB, RBLK, 0, G, fp32_stage).total + 1024;
-    int stages = (st_smem_budget(MB) - fixed) / st_stage_bytes(MB, RBLK);
+    int stages = (st_smem_budget(CTAS) - fixed) / st_stage_bytes(MB, RBLK);
     if (stages > ST_MAX_STAGES) stages = ST_MAX_STAGES;
     if (stages < 2) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)st_layout(MB, RBLK, stages, G, fp32_stage).total + 1024;
@@ -819,10 +819,10 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     static bool attr_done[64] = {false};
     static int resident[64] = {0};                          // CTAs of this instance that fit on the device at once
     if (!attr_done[dev]) {
-        e = cudaFuncSetAttribute(gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, st_smem_budget(MB));
+        e = cudaFuncSetAttribute(gemm_strip_kernel<MB, RBLK, DEBUG, FUSE, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, st_smem_budget(CTAS));
         if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, ST_THREADS, st_smem_budget(MB));
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE, CTAS>, ST_THREADS, st_smem_budget(CTAS));
         if (e != cudaSuccess) return e;
         resident[dev] = per_sm * device_sm_count();
         attr_done[dev] = true;
@@ -873,7 +873,7 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     attrs[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attrs;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE>, tm_act, tm_nib, tm_scale, tm_zero, a);
+    e = cudaLaunchKernelEx(&cfg, gemm_strip_kernel<MB, RBLK, DEBUG, FUSE, CTAS>, tm_act, tm_nib, tm_scale, tm_zero, a);
     if (e != cudaSuccess || FUSE != 2) return e;
     // two-kernel form: the requantisation once every maximum is final
     const int units = M * (N / 2 / GROUP);
@@ -883,7 +883,7 @@ cudaError_t launch_strip(const int8_t* qa, const uint16_t* sa, const int32_t* as
     return cudaLaunchKernelEx(&cfg, requant_kernel, (const __nv_bfloat16*)a.h, M, N / 2, a.qa_h, a.sa_h, a.asum_h, a.sync);
 }
 
-template <int MB, int RBLK>
+template <int MB, int RBLK, int CTAS>
 cudaError_t launch_strip_dbg(const int8_t* qa, const uint16_t* sa, const int32_t* asum, const void* packed, void* y,
                              const void* residual, void* y_copy, int M, int N, int K, int ctas, void* workspace,
                              int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
@@ -891,17 +891,17 @@ cudaError_t launch_strip_dbg(const int8_t* qa, const uint16_t* sa, const int32_t
         // two token blocks always run on 32-row strips (strip_plan): the other widths are not built in the fused form
         if constexpr (MB == 2 && RBLK != 2) return cudaErrorInvalidConfiguration;
         else if (fuse->one_kernel)
-            return launch_strip<MB, RBLK, false, 1>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
+            return launch_strip<MB, RBLK, false, 1, CTAS>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
         else
-            return launch_strip<MB, RBLK, false, 2>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
+            return launch_strip<MB, RBLK, false, 2, CTAS>(qa, sa, asum, packed, nullptr, nullptr, nullptr, M, N, K, ctas, workspace, nullptr, fuse, stream);
     }
     if (residual) {                                      // its own instantiation: the plain kernel's epilogue stays as small as it was
         if constexpr (MB == 2 && RBLK != 2) return cudaErrorInvalidConfiguration;
-        else return launch_strip<MB, RBLK, false, 3>(qa, sa, asum, packed, y, residual, nullptr, M, N, K, ctas, workspace, nullptr, nullptr, stream);
+        else return launch_strip<MB, RBLK, false, 3, CTAS>(qa, sa, asum, packed, y, residual, nullptr, M, N, K, ctas, workspace, nullptr, nullptr, stream);
     }
     if (debug_partials)
-        return launch_strip<MB, RBLK, true, 0>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, debug_partials, nullptr, stream);
-    return launch_strip<MB, RBLK, false, 0>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, nullptr, nullptr, stream);
+        return launch_strip<MB, RBLK, true, 0, CTAS>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, debug_partials, nullptr, stream);
+    return launch_strip<MB, RBLK, false, 0, CTAS>(qa, sa, asum, packed, y, nullptr, y_copy, M, N, K, ctas, workspace, nullptr, nullptr, stream);
 }
 
 }  // namespace
@@ -921,14 +921,13 @@ bool strip_supported(int M, int N, int K) {
 
 // Strip width and CTA count for a problem (measured on B200, sweep of widths 16..128 and 148..296 CTAs on the
 // four layer shapes of an 8B-class decoder, 4 to 16 tokens): the widest strip that still gives about 1.25 strips
-// per SM (one step narrower if a wide strip would leave SMs with a single CTA), and up to two CTAs per SM up to 8 tokens - the second CTA's warps multiply while the first one's wait for data, which is
+// per SM (one step narrower if a wide strip would leave SMs with a single CTA), and up to two CTAs per SM up to 8 tokens (for 9 to 16 see below) - the second CTA's warps multiply while the first one's wait for data, which is
 // worth more than a whole SM's shared memory held free for the next launch; the next launch's CTAs still start
 // (and prefetch) as soon as the first CTAs of this one leave.  Wide strips share an activation tile between more
 // rows (less traffic from L2 into shared memory); 16-row strips are left to up to 8 tokens, where their 16
 // activation tiles per stage still leave room for a ring.  The grid never exceeds the number of strips, so that a
 // strip is shared by at most two CTAs.
 void strip_plan(int M, int N, int K, int* strip_rows, int* ctas) {
-    (void)K;
     const int sms = device_sm_count();
     int R = 128;
     if (M <= 8) {
@@ -943,7 +942,13 @@ void strip_plan(int M, int N, int K, int* strip_rows, int* ctas) {
         if (v == 16 || v == 32 || v == 64 || v == 128) R = v;
     }
 #endif
-    int limit = st_ctas_per_sm(M <= 8 ? 1 : 2) * sms;
+    // Two token blocks: one CTA per SM, but two where that gives every strip a CTA of its own (no hand-over) at little cost in
+    // idle places.  Measured on B200 behind the quantiser at 16 tokens, one and two per SM: 192 strips K = 1024 5.5 and 5.2 us,
+    // 2048 6.7 and 6.8, 4096 9.0 and 9.5; 256 strips K = 1024 5.6 and 5.2, 2048 7.5 and 6.6, 3072 8.8 and 8.1, 4096 9.7 and 9.5; 160 strips
+    // K = 1024 5.4 and 5.3, 3072 7.4 and 7.9; more strips than places (384): K = 1024 6.8 and 7.2.
+    const int strips = N / R;
+    const bool two = M <= 8 || (strips > sms && strips <= 2 * sms && (long)K * (2 * sms - strips) <= 131072);
+    int limit = (two ? 2 : 1) * sms;
 #ifdef W4A8_TUNING
     if (const char* e = getenv("W4A8_STRIP_CTAS")) { const int v = atoi(e); if (v >= 1) limit = v; }
 #endif
@@ -961,18 +966,19 @@ cudaError_t strip_dispatch(const int8_t* qa, const uint16_t* sa, const int32_t* 
                            int32_t* debug_partials, const FuseOut* fuse, cudaStream_t stream) {
     int R = 0, ctas = 0;
     strip_plan(M, N, K, &R, &ctas);
-#define W4A8_STRIP_CASE(MBV, RBV) \
-    return launch_strip_dbg<MBV, RBV>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, ctas, workspace, debug_partials, fuse, stream)
+#define W4A8_STRIP_CASE(MBV, RBV, CTASV) \
+    return launch_strip_dbg<MBV, RBV, CTASV>(qa, sa, asum, packed, y, residual, y_copy, M, N, K, ctas, workspace, debug_partials, fuse, stream)
     if (M <= 8) {
-        if (R == 128) W4A8_STRIP_CASE(1, 8);
-        if (R == 64) W4A8_STRIP_CASE(1, 4);
-        if (R == 32) W4A8_STRIP_CASE(1, 2);
-        W4A8_STRIP_CASE(1, 1);
+        if (R == 128) W4A8_STRIP_CASE(1, 8, 2);
+        if (R == 64) W4A8_STRIP_CASE(1, 4, 2);
+        if (R == 32) W4A8_STRIP_CASE(1, 2, 2);
+        W4A8_STRIP_CASE(1, 1, 2);
     }
-    if (R == 128) W4A8_STRIP_CASE(2, 8);
-    if (R == 64) W4A8_STRIP_CASE(2, 4);
-    if (R == 32) W4A8_STRIP_CASE(2, 2);
-    W4A8_STRIP_CASE(2, 1);
+    if (R == 128) W4A8_STRIP_CASE(2, 8, 1);
+    if (R == 64) W4A8_STRIP_CASE(2, 4, 1);
+    if (R == 32 && ctas > device_sm_count()) W4A8_STRIP_CASE(2, 2, 2);
+    if (R == 32) W4A8_STRIP_CASE(2, 2, 1);
+    W4A8_STRIP_CASE(2, 1, 1);
 #undef W4A8_STRIP_CASE
 }
 }  // namespace

@@ -177,3 +177,19 @@ def test_separate_form_needs_its_scratch_and_shapes_are_checked():
     args[6] = 2 * I + 128                                       # N / 2 not a multiple of 128
     assert L.w4a8_gate_up_silu_quantize(*args) == B.ERR_SHAPE
     torch.cuda.synchronize()
+
+
+def test_auto_without_scratch_takes_the_epilogue_form():
+    """Layers whose rule says SEPARATE are accepted without a scratch up to 16 tokens, with the results of the epilogue form."""
+    M, K, I = 12, 256, 6144
+    c, packed = fused_layer(K, I, 6, M)
+    ws = B.new_workspace(M, 2 * I, K)
+    qa, sa, asum = B.w4a8_quantize_act(t_u16(c["x"], torch.bfloat16))
+    assert B.w4a8_gate_up_form(M, 2 * I, K) == B.GATE_UP_SEPARATE
+    want = B.w4a8_gate_up_silu_quantize(qa, sa, asum, packed, 2 * I, ws, form=B.GATE_UP_EPILOGUE)
+    got = B._h_outputs(M, I, 128, qa.device, None)
+    code = B.lib().w4a8_gate_up_silu_quantize(B.GATE_UP_AUTO, B._ptr(qa), B._ptr(sa), B._ptr(asum), B._ptr(packed), M, 2 * I, K, 128,
+                                              *(B._ptr(t) for t in got), None, B._ptr(ws), ws.numel(), B._stream(None))
+    assert code == B.OK
+    B.w4a8_check_status(ws)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))

@@ -1,6 +1,6 @@
-"""GPU parity of the strip kernel with two token blocks (9 to 16 tokens, one CTA per SM) where it can go wrong: fewer strips
-than SMs, strips shared by neighbouring CTAs, a ragged last stage, one group, and both sides of the rule that leaves a long K
-over few channels to the cluster kernel.  Partials D bit-exact, output within the band of the linear layer, residual form
+"""GPU parity of the strip kernel with two token blocks (9 to 16 tokens, one CTA per SM or one per strip) where it can go wrong: fewer strips
+than SMs, strips shared by neighbouring CTAs, a ragged last stage, one group, and both sides of the rules that leave a long K
+over few channels and a short one over many to the cluster kernel.  Partials D bit-exact, output within the band of the linear layer, residual form
 within its own."""
 import numpy as np
 import pytest
@@ -15,7 +15,7 @@ from tests.gpu_util import DeviceLayer, bits, t_u16
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("K,N,family", [(128, 128, B.PATH_STRIP), (2048, 1920, B.PATH_STRIP), (2176, 1920, B.PATH_SPLITK),
+@pytest.mark.parametrize("K,N,family", [(128, 128, B.PATH_STRIP), (2048, 1920, B.PATH_STRIP), (2176, 1920, B.PATH_SPLITK), (512, 5120, B.PATH_SPLITK), (640, 6144, B.PATH_STRIP), (1152, 8192, B.PATH_STRIP),
                                         (2176, 2048, B.PATH_STRIP), (4096, 4096, B.PATH_STRIP), (1152, 5120, B.PATH_STRIP),
                                         (6144, 4864, B.PATH_STRIP)])
 def test_two_token_blocks(K, N, family):

@@ -183,3 +183,14 @@ def test_tile_height_of_layers_with_few_groups():
                           (400, 24576, 1024, 208), (100, 8192, 1024, 64), (64, 24576, 1024, 64), (512, 8192, 512, 128), (700, 8192, 512, 208), (1024, 24576, 256, 208),
                           (300, 24576, 384, 128), (128, 1024, 512, 64)):
         assert B.w4a8_plan(M, N, K)["tile_m"] == tile, (M, N, K)
+
+
+def test_kernels_for_nine_to_sixteen_tokens():
+    """Both lines of the strip kernel's rule, and its CTAs: one per SM, or one per strip where that spares the hand-over."""
+    for N, K, family in ((1024, 128, B.PATH_SPLITK), (128, 128, B.PATH_STRIP), (4096, 256, B.PATH_STRIP), (24576, 256, B.PATH_SPLITK),
+                         (5120, 512, B.PATH_SPLITK), (5120, 768, B.PATH_STRIP), (12288, 1536, B.PATH_SPLITK), (12288, 2048, B.PATH_STRIP),
+                         (24576, 4096, B.PATH_STRIP), (2048, 28672, B.PATH_STRIP), (1024, 4096, B.PATH_SPLITK)):
+        assert B.w4a8_plan(16, N, K)["family"] == family and B.w4a8_plan(8, N, K)["family"] == B.PATH_STRIP, (N, K)
+    for N, K, ctas in ((6144, 1024, 192), (6144, 4096, 148), (8192, 2048, 256), (8192, 4096, 148), (5120, 4096, 148), (4096, 1024, 128)):
+        p = B.w4a8_plan(16, N, K)
+        assert p["ctas"] == ctas and p["strip_rows"] == 32, (N, K)
