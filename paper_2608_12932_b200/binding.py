@@ -357,8 +357,8 @@ def w4a8_linear(x, packed_w, N, workspace, group=GROUP, out=None, scratch=None, 
     else:
         _dev(out, torch.bfloat16, "out")
     if scratch is None:
-        # one allocation for the three: codes, group sums, token scales, each 16-byte aligned (K is a multiple of 128)
-        scales_at = M * K + 4 * M * (K // group)
+        # one allocation for the three: codes (16-byte aligned), group sums (the same, K being a multiple of 128), token scales
+        scales_at = M * K + 4 * M * max(K // group, 1)
         buf = torch.empty(scales_at + 2 * M, dtype=torch.uint8, device=x.device)
         qa = buf.data_ptr()
         sa, asum = qa + scales_at, qa + M * K

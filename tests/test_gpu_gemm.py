@@ -501,6 +501,16 @@ def test_linear_errors():
     assert y.shape == (0, case["N"])
 
 
+@pytest.mark.parametrize("group", [-128, -1, 32, 64, 256])
+def test_linear_refuses_other_group_sizes_with_a_status(group):
+    """Whatever the scratch would have measured for such a group: the library's own refusal, not an allocation error."""
+    case = wl.make_config("tiny")
+    layer = DeviceLayer(case, 16)
+    with pytest.raises(B.W4A8Error) as e:
+        B.w4a8_linear(t_u16(case["x"], torch.bfloat16), layer.packed, layer.N, layer.ws, group=group)
+    assert e.value.code == B.ERR_SHAPE
+
+
 def test_plan_matches_the_device():
     """On the GPU the planner may split K over a cluster when a problem has few tiles; whatever it
     picks fits the machine, and the result of the dispatch it describes is right."""
