@@ -308,8 +308,10 @@ def plan_name(B, M, N, K):
         return f"gemm_strip_kernel<{p['tile_m'] // 8},{p['strip_rows'] // 16}> x {p['ctas']} CTAs"
     if p["family"] == B.PATH_SPLITK:
         return f"gemm_cluster_kernel<{p['tile_m'] // 8}> x {p['ctas']} CTAs, {p['k_slices']} K slices"
-    name = "gemm_tcshort_kernel" if p["tile_m"] == 64 else "gemm_tcgen05_kernel"
-    return (f"{name}<{p['tile_m']}> x {p['ctas']} CTAs" + (f", {p['k_slices']} K slices" if p["k_slices"] > 1 else "")
+    # 64-row tiles: a kernel of their own, cut to 32 columns up to 32 tokens; layers of up to four groups keep the tall one's
+    short = p["tile_m"] == 64 and (M <= 32 or K > 512)
+    name, tile = ("gemm_tcshort_kernel", 32 if M <= 32 else 64) if short else ("gemm_tcgen05_kernel", p["tile_m"])
+    return (f"{name}<{tile}> x {p['ctas']} CTAs" + (f", {p['k_slices']} K slices" if p["k_slices"] > 1 else "")
             + (", balanced walk" if p["balanced"] else ""))
 
 
@@ -460,7 +462,7 @@ def run_rope_roofline(torch, B, peaks, l2_bytes, timer):
                 B.w4a8_rope_shifted_keys(k, pos, 45, 1.0e6, out=out)
         _, times = timer.graph_ms(body, replays=5, warm=2)
         us = float(np.median(times)) * 1e3 / ncopies
-        rows.append({"kernel": "rope_shifted_keys_kernel", "workload": f"T={T} H={H} D={D}", "bound": "hbm",
+        rows.append({"kernel": "rope_shifted_keys_wide_kernel" if T * H * D >= 4 << 20 else "rope_shifted_keys_kernel", "workload": f"T={T} H={H} D={D}", "bound": "hbm",
                      "achieved": round(nbytes / us / 1e3, 1), "unit": "GB/s", "peak": peaks["hbm_gbs"],
                      "frac": round(nbytes / us / 1e3 / peaks["hbm_gbs"], 4), "us_per_launch": round(us, 2),
                      "algorithmic_bytes_per_launch": nbytes})

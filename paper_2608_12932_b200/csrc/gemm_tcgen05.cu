@@ -115,7 +115,7 @@ struct Cfg {
     static constexpr int B_OFF = 0;
     static constexpr int RAW_OFF = B_OFF + SB * B_BYTES;
     static constexpr int BAR_OFF = RAW_OFF + SR * RAW_STRIDE;
-    static constexpr int NUM_BARS = 2 * SR + SB + SA + 4 + DONE_RING + 2 + 2;
+    static constexpr int NUM_BARS = 2 * SR + SB + SA + NB + DONE_RING + 2 + 2;
     static constexpr int MISC_OFF = (BAR_OFF + NUM_BARS * 8 + 15) & ~15;      // 16-byte aligned: staging is read with 16-byte loads
     static constexpr int W = TILE_M / 2;                                      // accumulator columns (tokens) per drain warp
     static constexpr int NCH = (W + 31) / 32;                                 // 32-column chunks per drain warp (the last may be 8 wide)
@@ -178,7 +178,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     // one event frees the step's weight stage (unpack warps wait for step it - SA), its activation
     // stage (producer waits for step it - SB) and publishes its accumulator (drain warps wait for it).
     const int RAW_FULL = 0, RAW_EMPTY = C::SR, B_FULL = 2 * C::SR, A_FULL = B_FULL + C::SB, ACC_EMPTY = A_FULL + C::SA,
-              DONE = ACC_EMPTY + 4, FINAL = DONE + DONE_RING, TILE_DONE = FINAL + 2;
+              DONE = ACC_EMPTY + C::NB, FINAL = DONE + DONE_RING, TILE_DONE = FINAL + 2;
     auto done_bar = [&](uint32_t step) { return bar(DONE + (int)(step % DONE_RING)); };
     auto done_parity = [](uint32_t step) { return (step / DONE_RING) & 1u; };
     volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem + C::MISC_OFF);
@@ -193,7 +193,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             }
             for (int i = 0; i < C::SB; ++i) ptx::mbar_init(bar(B_FULL + i), 1);
             for (int i = 0; i < C::SA; ++i) ptx::mbar_init(bar(A_FULL + i), NUM_UNPACK_WARPS);
-            for (int i = 0; i < 4; ++i) ptx::mbar_init(bar(ACC_EMPTY + i), NUM_DRAIN_WARPS);
+            for (int i = 0; i < C::NB; ++i) ptx::mbar_init(bar(ACC_EMPTY + i), NUM_DRAIN_WARPS);
             for (int i = 0; i < DONE_RING; ++i) ptx::mbar_init(bar(DONE + i), 1);
             for (int i = 0; i < 2; ++i) ptx::mbar_init(bar(FINAL + i), 1);
             for (int i = 0; i < 2; ++i) ptx::mbar_init(bar(TILE_DONE + i), 2);      // both MMA issuers
@@ -438,7 +438,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             __syncwarp();
         }
         if (lane == 0) {                                          // the accumulator buffers start out free
-            for (int i = 0; i < 4; ++i) ptx::mbar_arrive(bar(ACC_EMPTY + i));
+            for (int i = 0; i < C::NB; ++i) ptx::mbar_arrive(bar(ACC_EMPTY + i));
         }
         uint32_t it = 0, tcount = 0;
         bool ok = true;
