@@ -31,6 +31,8 @@ constexpr int ROPE_WARPS = 8;
 constexpr int ROPE_MAX_HALF = 128;
 struct RopeTheta { double t[ROPE_MAX_HALF]; };               // theta_i / pi
 
+// The 4-byte form's angle and rotation: the operations of the wide form, each multiply-add as the compiler contracts it there
+// (the wide form spells them out in place; through these functions it is 0.5 to 1 % slower: 32768 x 8 x 128 25.2 and 25.5 us).
 // (cos, sin) of q theta_i
 __device__ __forceinline__ float2 rope_cos_sin(double q, double theta_over_pi) {
     const double a = __dmul_rn(q, theta_over_pi);
@@ -43,7 +45,7 @@ __device__ __forceinline__ void rope_rotate2(uint32_t& x, uint32_t& y, float c0,
     const float x0 = __uint_as_float(x << 16), x1 = __uint_as_float(x & 0xFFFF0000u);
     const float y0 = __uint_as_float(y << 16), y1 = __uint_as_float(y & 0xFFFF0000u);
     x = ptx::pack_bf16x2(fmaf(x0, c0, -__fmul_rn(y0, s0)), fmaf(x1, c1, -__fmul_rn(y1, s1)));
-    y = ptx::pack_bf16x2(fmaf(y0, c0, __fmul_rn(x0, s0)), fmaf(y1, c1, __fmul_rn(x1, s1)));
+    y = ptx::pack_bf16x2(fmaf(x0, s0, __fmul_rn(y0, c0)), fmaf(x1, s1, __fmul_rn(y1, c1)));
 }
 
 // TABLE: theta from the host; otherwise (longer half rows) from base ^ (-2 i / D) here.  Eight heads at a time, the rest by
@@ -133,21 +135,33 @@ rope_shifted_keys_wide_kernel(const uint4* __restrict__ k_pre, const int32_t* __
         }
         if (base == 0) {
             const double q = (double)(p - delta);
-            for (int i = lane; i < half; i += 32) rot[warp][i] = rope_cos_sin(q, th[i]);
+            for (int i = lane; i < half; i += 32) {
+                double a = q * th[i];
+                a -= 2.0 * rint(0.5 * a);
+                float2 cs;
+                sincospif((float)a, &cs.y, &cs.x);
+                rot[warp][i] = cs;
+            }
             __syncwarp();
         }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             if (base + lane + 32 * k < total) {
                 const float4* cs = reinterpret_cast<const float4*>(&rot[warp][8 * w[k]]);
-                uint32_t xs[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w}, ys[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
+                uint32_t ox[4], oy[4];
+                const uint32_t xs[4] = {lo[k].x, lo[k].y, lo[k].z, lo[k].w}, ys[4] = {hi[k].x, hi[k].y, hi[k].z, hi[k].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float4 c = cs[e];                  // cos, sin of element 2 e, then of 2 e + 1
-                    rope_rotate2(xs[e], ys[e], c.x, c.y, c.z, c.w);
+                    const float x0 = __uint_as_float(xs[e] << 16), x1 = __uint_as_float(xs[e] & 0xFFFF0000u);
+                    const float y0 = __uint_as_float(ys[e] << 16), y1 = __uint_as_float(ys[e] & 0xFFFF0000u);
+                    const __nv_bfloat162 olo = __floats2bfloat162_rn(x0 * c.x - y0 * c.y, x1 * c.z - y1 * c.w);
+                    const __nv_bfloat162 ohi = __floats2bfloat162_rn(y0 * c.x + x0 * c.y, y1 * c.z + x1 * c.w);
+                    ox[e] = *reinterpret_cast<const uint32_t*>(&olo);
+                    oy[e] = *reinterpret_cast<const uint32_t*>(&ohi);
                 }
-                k_rot[at[k]] = make_uint4(xs[0], xs[1], xs[2], xs[3]);
-                k_rot[at[k] + pieces] = make_uint4(ys[0], ys[1], ys[2], ys[3]);
+                k_rot[at[k]] = make_uint4(ox[0], ox[1], ox[2], ox[3]);
+                k_rot[at[k] + pieces] = make_uint4(oy[0], oy[1], oy[2], oy[3]);
             }
         }
     }
@@ -173,8 +187,10 @@ cudaError_t launch_rope_shifted_keys(const void* k_pre, const int32_t* pos, int 
     const double log2_base = log2(base);
     RopeTheta theta;
     for (int i = 0; table && i < D / 2; ++i) theta.t[i] = exp2(-(double)(2 * i) / (double)D * log2_base) * 0.31830988618379067154;
-    // measured on B200 (cold keys, 4-byte -> wide form): 30000 x 16 x 64 35.8 -> 21.6 us, 16384 x 8 x 128 15.4 -> 13.7, 65536 x 8 x 128
-    // 48.5 -> 47.8; 2000 x 8 x 128 3.6 -> 4.4 (one wave of CTAs: the shorter latency chain of the 4-byte form wins)
+    // Measured on B200 (cold keys, 4-byte and wide form, us, back to back in a graph): 16384 x 8 x 64 10.6 and 7.9, 16384 x 16 x 64 15.6
+    // and 11.3, 32768 x 16 x 32 27.7 and 13.0, 8192 x 4 x 128 6.2 and 5.3, 2048 x 8 x 128 3.4 and 4.4.  From 8 Mi elements of D = 128 on,
+    // where a half row fills a warp of 4-byte accesses, the 4-byte kernel itself is the quicker one (16384 x 8 x 128 11.3 and 13.3), but
+    // not in a stream of eager calls, where it does not start under its predecessor (14.6 and 14.2).
     if ((long long)T * H * D >= ROPE_WIDE_MIN_ELEMENTS && D % 16 == 0 && table && ((reinterpret_cast<uintptr_t>(k_pre) | reinterpret_cast<uintptr_t>(k_rot)) & 15) == 0) {
         cudaLaunchConfig_t cfg = {};
         cfg.stream = stream;

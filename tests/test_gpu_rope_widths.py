@@ -35,7 +35,7 @@ def test_widths_and_alignments(T, H, D, offset):
     assert np.all(np.abs(onp.bf16_bits_to_f64(out) - ref) <= bound)
 
 
-@pytest.mark.parametrize("T,H,D", [(4096, 8, 128), (5461, 3, 256), (16384, 16, 16)])
+@pytest.mark.parametrize("T,H,D", [(4096, 8, 128), (5461, 3, 256), (16384, 16, 16), (8193, 8, 128), (12000, 11, 64), (5462, 3, 256)])
 def test_a_key_does_not_depend_on_the_window_around_it(T, H, D):
     """A window of 4 Mi elements takes the 16-byte form, its parts the 4-byte one: the same bits for the same key."""
     rng = np.random.default_rng(D)
