@@ -192,7 +192,7 @@ w4a8_status w4a8_gemm_residual(w4a8_path path, const int8_t* qa, const uint16_t*
  *   y_gate_up  device, bf16 [M, 2 I] in the layout above (16-byte aligned)
  *   h          device, bf16 [M, I], receives h; may be NULL
  *   qa_h       device, int8 [M, I]; sa_h fp16 [M]; asum_h int32 [M, I / 128]
- *   I % 128 == 0, group == 128.  One kernel: one CTA per token, or a cluster of CTAs per token for few tokens.
+ *   I % 128 == 0, group == 128.  One kernel: one CTA per token, or a cluster of CTAs per token for few tokens and a large I.
  *
  * w4a8_gate_up_silu_quantize: projection and step together, in one of three forms (results identical bit for bit):
  *   W4A8_GATE_UP_EPILOGUE    the strip kernel's epilogue forms h from its own sums, stores it and keeps each token's
