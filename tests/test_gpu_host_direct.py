@@ -45,3 +45,28 @@ def test_new_inputs_in_the_same_buffers_and_the_device_copies(M, K, N):
         torch.cuda.synchronize()
         assert np.array_equal(y.view(torch.int16).numpy().view(np.uint16), want)
         assert np.array_equal(bits(linear.x_dev), x_bits) and np.array_equal(bits(linear.y_dev), want)
+
+
+@pytest.mark.parametrize("M,K,N", [(8, 1024, 6144), (40, 1024, 512)])
+def test_captured_into_a_graph(M, K, N):
+    """The questions to the driver about the host buffers are asked at capture; a replay reads what the buffer holds then."""
+    case = wl.make_layer(K, N, 95 + M, 2 * M)
+    layer = DeviceLayer(case, M)
+    linear = B.HostLinear(M, N, K, layer.packed, layer.ws)
+    x = torch.zeros((M, K), dtype=torch.bfloat16).pin_memory()
+    y = torch.empty((M, N), dtype=torch.bfloat16).pin_memory()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        linear(x, y)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        linear(x, y)
+    for i in range(2):
+        x_bits = case["x"][i * M:(i + 1) * M]
+        want = bits(B.w4a8_linear(t_u16(x_bits, torch.bfloat16), layer.packed, N, layer.ws))
+        x.view(torch.int16).copy_(torch.from_numpy(x_bits.view(np.int16)))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(y.view(torch.int16).numpy().view(np.uint16), want)
+        assert np.array_equal(bits(linear.x_dev), x_bits) and np.array_equal(bits(linear.y_dev), want)
