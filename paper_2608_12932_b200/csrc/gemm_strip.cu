@@ -242,7 +242,11 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
     const int stages = a.stages, sps = a.sps;
     constexpr bool SILU = FUSE == 1 || FUSE == 2;          // gate+up epilogue; FUSE == 3: residual epilogue
     const StLayout L = st_layout(MB, RBLK, stages, G, FUSE == 3);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // The warp index comes out of a shuffle, so that the compiler knows it to be warp-uniform: the roles' loop counters, ring and
+    // barrier addresses then live on the uniform datapath.  (B200, one launch behind another, cold weights, before and after:
+    // 4096 -> 24576 at 1, 8 and 16 tokens 13.8, 13.7 and 17.8 us, 13.3, 13.1 and 16.8; 4096 -> 6144 at 8 5.1, 4.8; 12288 -> 4096 with
+    // residual at 8 and 16 7.9 and 10.3, 7.5 and 9.6; warp instructions of the first at 8 tokens 5.69 M, 5.37 M.)
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
 
     // this CTA's contiguous range of stages, [lo, hi), and the strips it touches
     const int lo = (int)(((long long)blockIdx.x * a.total_stages) / gridDim.x);

@@ -112,7 +112,10 @@ gemm_tcshort_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
     const int GK = K / GROUP;                                   // groups of the whole K range (blob and output indexing)
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // The warp index comes out of a shuffle: the compiler then knows it to be warp-uniform and keeps ring indices, barrier and
+    // tensor-memory addresses on the uniform datapath (B200, before and after: 4096 -> 24576 at 40 and 64 tokens 19.7 and 19.9 us, 18.9
+    // and 19.2; 4096 -> 6144 at 40 9.7, 9.4).
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     const int slice = SPLIT ? (int)ptx::cluster_ctarank() : 0;
     const int unit = SPLIT ? (int)blockIdx.x / S : (int)blockIdx.x;
     const int num_units = SPLIT ? (int)gridDim.x / S : (int)gridDim.x;
