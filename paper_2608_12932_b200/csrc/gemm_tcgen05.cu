@@ -8,7 +8,7 @@
 // Orientation ("swap-AB"): the 128 output channels of a tile are the MMA's M side (TMEM lanes),
 // the tokens are its N side (TMEM columns).  A drain thread therefore owns ONE output channel:
 // its group scale is a per-thread scalar and the per-group work on the CUDA cores is one
-// int->float convert and one FMA per accumulator element.
+// int->float convert and half a packed FMA per accumulator element.
 //
 // One pipeline step = one quantisation group = 128 k = four K=32 MMAs; the accumulator must be
 // drained after every group because the scale changes, so TMEM holds two accumulator buffers:
@@ -35,6 +35,15 @@
 //    three barrier waits, four MMAs and a commit); the whole warp walks the loop and an elected lane
 //    issues, which keeps the MMA operands in uniform registers (from inside a one-lane branch every
 //    MMA cost its thread about a hundred cycles of register-to-uniform moves);
+//  * what paces a step of a 208-row tile is the chain of a drain warp - the look at its barrier, the loads, the hand-back and the
+//    sums, 100 to 200 cycles for each of the first three however long ago the MMAs finished (measured with stamps; the
+//    barrier has completed at the first look five times out of six).  So the warp index is made warp-uniform (ring indices,
+//    barrier and tensor-memory addresses on the uniform datapath), arrivals are predicated instructions instead of one-lane
+//    branches, the next step's barrier is looked at under the loads, and two sums take one packed FMA: 4096 -> 24576 at 1024
+//    and 4096 tokens 132.4 and 523 us before, 125.4 and 491 after, 4096 -> 6144 40.2 and 132, 38.3 and 125.7; with a residual
+//    0 to 4 % (B200, weights cold).  Tried on top, none quicker: the conversion moved to the FMA pipe by a constant bias in the
+//    accumulators (131), for half of the columns (134), the two halves of the columns filled and handed back on their own (144),
+//    columns loaded in pieces ahead of the sums (129.6), a tile's outputs staged whole (127.4 before the look ahead, equal);
 //  * one tcgen05.commit per step, on a ring of "step done" barriers, frees the step's weight and
 //    activation stages and publishes its accumulator.
 //
@@ -165,7 +174,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
     const int GK = K / GROUP;                                   // groups of the whole K range (blob and output indexing)
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);     // known to be warp-uniform this way: see the header
     // SPLIT: a cluster of S CTAs per tile (one tile per cluster, no persistence); this CTA walks groups [g_lo, g_lo + G)
     const int slice = SPLIT ? (int)ptx::cluster_ctarank() : 0;
     const int unit = SPLIT ? (int)blockIdx.x / S : (int)blockIdx.x;
@@ -410,10 +420,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) {
-                    ptx::mbar_arrive(bar(A_FULL + sa_));
-                    ptx::mbar_arrive(bar(RAW_EMPTY + sr));
-                }
+                ptx::mbar_arrive_if(bar(A_FULL + sa_), lane == 0);
+                ptx::mbar_arrive_if(bar(RAW_EMPTY + sr), lane == 0);
             }
         }
     } else {
@@ -441,7 +449,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             for (int i = 0; i < C::NB; ++i) ptx::mbar_arrive(bar(ACC_EMPTY + i));
         }
         uint32_t it = 0, tcount = 0;
-        bool ok = true;
+        bool ok = true, ready = false;                            // ready: step `it` is known to be complete
         // token scales (raw fp16 bits) and first group scale of the next segment, requested before the epilogue of
         // the current one so that their latency is not added to the time the tensor pipe waits for this warp
         uint16_t next_sa_bits[C::NCH], next_sw_bits = 0;
@@ -468,9 +476,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             const int n = ntile * TILE_N + n_local;
             const int m_base = mtile * TILE_M + h * C::W;
             const uint8_t* sw_ptr = packed + ((size_t)ntile * GK + g_lo) * BLOB_BYTES + BLOB_SCALE_OFF + 2 * n_local;
-            float facc[C::W];
+            uint64_t facc[C::W / 2];                              // pairs of neighbouring tokens
 #pragma unroll
-            for (int i = 0; i < C::W; ++i) facc[i] = 0.0f;
+            for (int i = 0; i < C::W / 2; ++i) facc[i] = 0ull;
+            auto sum = [&](int i) { const float2 t = ptx::unpack2(facc[i / 2]); return i & 1 ? t.y : t.x; };
             if (BAL && ge < G) {
                 // Balanced walk: this CTA's last tile, whose later groups the next CTA summed first (they open its range): the sums
                 // start from those.  Fetched here and not after the last group they are off the tail that the launch ends with,
@@ -480,7 +489,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 if (!ok) break;
                 const float* slot = handover + (size_t)(blockIdx.x + 1) * (TILE_M * TILE_N);
 #pragma unroll
-                for (int i = 0; i < C::W; ++i) facc[i] = __ldcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local);
+                for (int i = 0; i < C::W; i += 2) {
+                    const float* p = slot + (size_t)(h * C::W + i) * TILE_N + n_local;
+                    facc[i / 2] = ptx::pack2(__float_as_uint(__ldcg(p)), __float_as_uint(__ldcg(p + TILE_N)));
+                }
                 __syncwarp();
                 // this warp's bit back to zero for the next call
                 if (lane == 0) atomicAnd(handover_flags + blockIdx.x + 1, ~(1u << (warp - WARP_DRAIN0)));
@@ -524,14 +536,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
 #pragma unroll
                 for (int ch = 0; ch < C::NCH; ++ch) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
+                    for (int i = 0; i < 32; i += 2) {
                         if (ch * 32 + i < C::W) {
-                            const int32_t di = (int32_t)v[ch][i];
+                            const int32_t d0 = (int32_t)v[ch][i], d1 = (int32_t)v[ch][i + 1];
                             // exact while |sum| < 2^24; beyond that one rounding of relative size 2^-24
-                            facc[ch * 32 + i] = sw * (float)di;
+                            facc[(ch * 32 + i) / 2] = ptx::pack2(__float_as_uint(sw * (float)d0), __float_as_uint(sw * (float)d1));
                             if (DEBUG) {
                                 const int m = m_base + ch * 32 + i;
-                                if (m < M) debug_partials[(size_t)m * N + n] = di;
+                                if (m < M) debug_partials[(size_t)m * N + n] = d0;
+                                if (m + 1 < M) debug_partials[(size_t)(m + 1) * N + n] = d1;
                             }
                         }
                     }
@@ -540,10 +553,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             for (int g = gb; g < (PC ? gb : ge); ++g, ++it) {
                 const uint32_t buf = it & (C::NB - 1);
                 const float sw = __half2float(__ushort_as_half(sw_bits));
+                const uint64_t sw2 = ptx::pack2(__float_as_uint(sw), __float_as_uint(sw));
                 if (g + 1 < ge) sw_bits = __ldg(reinterpret_cast<const uint16_t*>(sw_ptr + (size_t)(g + 1) * BLOB_BYTES));
                 // (short tiles: this warp mostly waits, and a polling loop's probes queue up in front of the unpack
                 // warp's shared-memory accesses on the same scheduler; the parking wait leaves the queue alone)
-                if (!(ok = (TILE_M <= 128 ? ptx::mbar_wait(done_bar(it), done_parity(it), abort_flag)
+                if (!ready &&
+                    !(ok = (TILE_M <= 128 ? ptx::mbar_wait(done_bar(it), done_parity(it), abort_flag)
                                           : ptx::mbar_wait_hot(done_bar(it), done_parity(it), abort_flag)))) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t taddr = lane_taddr + buf * TILE_M;
@@ -556,20 +571,22 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                     if (ch == C::NCH - 1 && C::LAST == 8) ptx::tmem_ld_32x8(taddr + ch * 32, reinterpret_cast<uint32_t(&)[8]>(v[ch]));
                     else ptx::tmem_ld_32x32(taddr + ch * 32, v[ch]);
                 }
+                // the next step's barrier, looked at under the loads' latency (past the last step: a phase that never completes)
+                ready = ptx::mbar_test_wait(done_bar(it + 1), done_parity(it + 1));
                 ptx::tmem_ld_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(ACC_EMPTY + buf));
+                ptx::mbar_arrive_if(bar(ACC_EMPTY + buf), lane == 0);
 #pragma unroll
                 for (int ch = 0; ch < C::NCH; ++ch) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
+                    for (int i = 0; i < 32; i += 2) {
                         if (ch * 32 + i < C::W) {
-                            const int32_t di = (int32_t)v[ch][i];
-                            facc[ch * 32 + i] = fmaf(sw, (float)di, facc[ch * 32 + i]);     // exact convert: |D| < 2^24
+                            ptx::cvt_fma2(facc[(ch * 32 + i) / 2], v[ch][i], v[ch][i + 1], sw2);        // exact converts: |D| < 2^24
                             if (DEBUG) {
                                 const int m = m_base + ch * 32 + i;
-                                if (m < M) debug_partials[((size_t)m * GK + g_lo + g) * N + n] = di;
+                                if (m < M) debug_partials[((size_t)m * GK + g_lo + g) * N + n] = (int32_t)v[ch][i];
+                                if (m + 1 < M) debug_partials[((size_t)(m + 1) * GK + g_lo + g) * N + n] = (int32_t)v[ch][i + 1];
                             }
                         }
                     }
@@ -583,7 +600,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 // t * 128 + n of this CTA's slot, then this warp's bit of the slot's flag word (release).
                 float* slot = handover + (size_t)blockIdx.x * (TILE_M * TILE_N);
 #pragma unroll
-                for (int i = 0; i < C::W; ++i) __stcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local, facc[i]);
+                for (int i = 0; i < C::W; ++i) __stcg(slot + (size_t)(h * C::W + i) * TILE_N + n_local, sum(i));
                 __syncwarp();
                 if (lane == 0) ptx::red_or_release_gpu_u32(handover_flags + blockIdx.x, 1u << (warp - WARP_DRAIN0));
                 continue;                       // the other CTA stores the tile
@@ -605,7 +622,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                         const int owner = (run >= lo1) + (run >= lo2) + (run >= lo3);
                         const int first = run >= lo3 ? lo3 : (run >= lo2 ? lo2 : (run >= lo1 ? lo1 : 0));
                         const uint32_t at = smem_base + C::B_OFF + (uint32_t)((slice * runs_max + run - first) * TILE_N + slot_n) * 16u;
-                        ptx::st_dsmem_f32x4(ptx::map_to_cta(at, (uint32_t)owner), make_float4(facc[i], facc[i + 1], facc[i + 2], facc[i + 3]));
+                        ptx::st_dsmem_f32x4(ptx::map_to_cta(at, (uint32_t)owner), make_float4(sum(i), sum(i + 1), sum(i + 2), sum(i + 3)));
                     }
                 }
                 // This CTA's share, by the drain warps: a warp takes a run at a time (four tokens x the tile's 128 channels, four
@@ -718,7 +735,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                         for (int i = 0; i < 16; ++i)
                             if (b2 * 32 + 16 * half + i < C::W)
                                 reinterpret_cast<__nv_bfloat16*>(ob + (16 * half + i) * 64)[lane] =
-                                    __float2bfloat16_rn(facc[b2 * 32 + 16 * half + i] * sc[16 * half + i] + rs[i]);
+                                    __float2bfloat16_rn(sum(b2 * 32 + 16 * half + i) * sc[16 * half + i] + rs[i]);
                     }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) rv[k] = rv_next[k];
@@ -728,7 +745,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
                     if (b2 * 32 + i < C::W)
-                        reinterpret_cast<__nv_bfloat16*>(ob + i * 64)[lane] = __float2bfloat16_rn(facc[b2 * 32 + i] * sc[i]);
+                        reinterpret_cast<__nv_bfloat16*>(ob + i * 64)[lane] = __float2bfloat16_rn(sum(b2 * 32 + i) * sc[i]);
                 }
                 if (b2 < C::NCH - 1 || C::LAST == 32) {
                     // a full block of 32 tokens: one TMA store (rows past M are clipped by the map), the warp moves on

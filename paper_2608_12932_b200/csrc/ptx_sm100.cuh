@@ -119,6 +119,10 @@ constexpr uint32_t PARK_NS = 20000;                  // longest single park
 #define W4A8_WAIT_BACKOFF_NS 40
 #endif
 constexpr uint32_t WAIT_BACKOFF_NS = W4A8_WAIT_BACKOFF_NS;
+// arrival of the lanes with `go`, as a predicated instruction (a one-lane branch costs the warp its reconvergence)
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool go) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)go) : "memory");
+}
 // non-blocking probe of a phase (try_wait may suspend the thread for a while; this never does)
 __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -313,6 +317,14 @@ __device__ __forceinline__ void add_fma2(uint64_t& acc, uint32_t lo, uint32_t hi
         "add.rn.f32x2 t, t, %3;\n\t"
         "fma.rn.f32x2 %0, t, %4, %0;\n\t}"
         : "+l"(acc) : "r"(lo), "r"(hi), "l"(b), "l"(s));
+}
+// acc += float(v) * s for a pair of integers below 2^24
+__device__ __forceinline__ void cvt_fma2(uint64_t& acc, uint32_t lo, uint32_t hi, uint64_t s) {
+    asm("{\n\t.reg .b64 t;\n\t.reg .f32 x, y;\n\t"
+        "cvt.rn.f32.s32 x, %1;\n\tcvt.rn.f32.s32 y, %2;\n\t"
+        "mov.b64 t, {x, y};\n\t"
+        "fma.rn.f32x2 %0, t, %3, %0;\n\t}"
+        : "+l"(acc) : "r"(lo), "r"(hi), "l"(s));
 }
 
 // ---- tcgen05 ----------------------------------------------------------------------------------
