@@ -181,7 +181,7 @@ struct StripArgs {
     __nv_bfloat16* y_copy;   // null, or a second place for y (the plain form only)
     int M, N, K;
     int stages;              // ring length
-    int pre;                 // ring slots whose weights are requested before griddepcontrol.wait (the rest: L2 prefetch).
+    int pre;                 // ring slots whose weights are requested before griddepcontrol.wait.
                              // The whole ring: fewer (1..3 slots, so that the first activation tile would not queue behind
                              // them) changed nothing on the wide layers and cost 2 to 19 % on the narrow ones - the first
                              // tile takes 1.5-2 us under the weight stream however little this CTA has in flight.
@@ -300,20 +300,10 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
         // weights do not depend on the previous kernel: start their stream at once
         const int first = n < a.pre ? n : a.pre;
         for (int i = pw; i < first; i += ST_PRODUCER_WARPS) load_weights(lo + i, i);
-        // what the ring cannot hold is asked into L2 meanwhile, so that HBM keeps streaming under the previous
-        // kernel and the ring refills from L2 (a third of the latency) once this one runs
-        for (int i = first + pw; i < n; i += ST_PRODUCER_WARPS) {
-            const int t = lo + i, strip = t / sps, sg = t - strip * sps;
-            const int tile = strip / STRIPS_PER_TILE, r0 = (strip % STRIPS_PER_TILE) * R, g0 = sg * GS;
-            if (WHOLE) {
-                const int valid = (G - g0) < GS ? (G - g0) : GS;
-                ptx::bulk_prefetch_l2(a.packed + ((size_t)tile * G + g0) * BLOB_BYTES, (uint32_t)valid * BLOB_BYTES);
-            } else {
-                ptx::tma_prefetch_4d(&tm_nib, 0, r0, g0, tile);
-                ptx::tma_prefetch_3d(&tm_scale, r0, g0, tile);
-                ptx::tma_prefetch_3d(&tm_zero, R < 32 ? (r0 >> 5) * 16 : r0 / 2, g0, tile);
-            }
-        }
+        // (What the ring cannot hold is not asked into L2 meanwhile: requests for a whole layer at once delay the kernel that this one
+        // waits for - the quantiser, or the last stores of the projection before - by more than they bring.  4096 -> 24576 at 1, 8 and
+        // 16 tokens behind one another 13.2, 13.2 and 16.7 us with such requests, 11.5, 11.4 and 13.8 without; 12288 -> 4096 with
+        // residual at 16 9.5 and 8.7; behind the quantiser the same layer 15.7 and 13.7 at 8 tokens, 12288 -> 4096 10.1 and 10.4.)
     }
     // Activations, their scales and group sums, and the workspace belong to the previous kernel until
     // this wait returns.  They are read only after it and only through L2 (TMA, ld.global.cg).
