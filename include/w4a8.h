@@ -75,7 +75,8 @@ size_t w4a8_packed_bytes(int N, int K, int group);
  * per-tile arrival counters and hand-over flags; the strip kernel's hand-over slots; one status
  * word); 0 for an unsupported shape.  The first W4A8_WORKSPACE_ZEROED_BYTES bytes (or the whole
  * workspace, if it is smaller) must be zero before the first call (w4a8_workspace_init does that)
- * and are left zero by every call, so one workspace can serve any number of calls that do not
+ * and are left by every call as the next one needs them (zero, but for the fused gate+up call's
+ * maxima, which carry the numbers of their calls), so one workspace can serve any number of calls that do not
  * overlap on the GPU.
  */
 #define W4A8_WORKSPACE_HEADER_BYTES 4096

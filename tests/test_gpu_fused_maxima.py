@@ -1,0 +1,45 @@
+"""The per-token maxima that the fused gate+up call keeps in the workspace between its projection and its requantisation are never
+cleared: each call's supersede the last call's.  So a workspace that has served calls with larger values, other token
+counts and the other form gives the bits of a fresh one."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import w4a8_oracle as onp
+from paper_2608_12932_b200 import binding as B
+from paper_2608_12932_b200 import workload as wl
+from tests.gpu_util import bits, t_u16
+
+pytestmark = pytest.mark.gpu
+
+
+def bf16_bits(a):
+    return bits(torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().bfloat16())
+
+
+@pytest.mark.parametrize("M", [1, 8, 16])
+def test_a_used_workspace_gives_the_bits_of_a_fresh_one(M):
+    I, K = 256, 256
+    case = wl.make_layer(K, 2 * I, 11, 4)
+    packed = B.w4a8_pack_weights(torch.from_numpy(case["qw"]).cuda(), t_u16(case["sw"], torch.float16), torch.from_numpy(case["z"]).cuda())
+    rng = np.random.default_rng(5)
+    used = B.new_workspace(16, 2 * I, K)
+
+    def call(x_bits, ws, form):
+        q = B.w4a8_quantize_act(t_u16(x_bits, torch.bfloat16))
+        out = B.w4a8_gate_up_silu_quantize(*q, packed, 2 * I, ws, form=form)
+        B.w4a8_check_status(ws)
+        return out
+
+    small = rng.standard_normal((M, K)) * 0.01
+    small[M // 2] = 0.0                                        # a token whose h is zero throughout: no maximum is ever written
+    small = bf16_bits(small)
+    for form in (B.GATE_UP_EPILOGUE, B.GATE_UP_ONE_KERNEL, B.GATE_UP_EPILOGUE, B.GATE_UP_ONE_KERNEL):
+        call(bf16_bits(rng.standard_normal((16, K)) * 100.0), used, form)
+        for repeat in range(2):
+            got, fresh = call(small, used, form), call(small, B.new_workspace(16, 2 * I, K), form)
+            for a, b in zip(got, fresh):
+                assert torch.equal(a.view(torch.uint8) if a.dtype != torch.int32 else a, b.view(torch.uint8) if b.dtype != torch.int32 else b)
+            qa, sa, asum = onp.quantize_act(bits(got[0]), 128)
+            assert np.array_equal(got[1].cpu().numpy(), qa) and np.array_equal(bits(got[2]), sa) and np.array_equal(got[3].cpu().numpy(), asum)
+            assert bits(got[2])[M // 2] == 0
