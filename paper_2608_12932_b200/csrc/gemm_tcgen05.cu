@@ -519,7 +519,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 // one drain per tile: the buffer holds the sum of D over all groups (|sum| < 2^31 for K < 2^13 * 128)
                 const uint32_t buf = tcount & 1u;
                 const float sw = __half2float(__ushort_as_half(sw_bits));
-                if (!(ok = ptx::mbar_wait_hot(bar(TILE_DONE + buf), (tcount >> 1) & 1, abort_flag))) break;
+                if (!(ok = ptx::warp_mbar_wait_hot(bar(TILE_DONE + buf), (tcount >> 1) & 1, abort_flag))) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t taddr = lane_taddr + buf * TILE_M;
                 uint32_t v[C::NCH][32];
@@ -558,8 +558,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 // (short tiles: this warp mostly waits, and a polling loop's probes queue up in front of the unpack
                 // warp's shared-memory accesses on the same scheduler; the parking wait leaves the queue alone)
                 if (!ready &&
-                    !(ok = (TILE_M <= 128 ? ptx::mbar_wait(done_bar(it), done_parity(it), abort_flag)
-                                          : ptx::mbar_wait_hot(done_bar(it), done_parity(it), abort_flag)))) break;
+                    !(ok = (TILE_M <= 128 ? ptx::warp_mbar_wait(done_bar(it), done_parity(it), abort_flag)
+                                          : ptx::warp_mbar_wait_hot(done_bar(it), done_parity(it), abort_flag)))) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t taddr = lane_taddr + buf * TILE_M;
                 // All of this warp's columns go to registers with back-to-back loads, then the buffer is
@@ -572,7 +572,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                     else ptx::tmem_ld_32x32(taddr + ch * 32, v[ch]);
                 }
                 // the next step's barrier, looked at under the loads' latency (past the last step: a phase that never completes)
-                ready = ptx::mbar_test_wait(done_bar(it + 1), done_parity(it + 1));
+                ready = ptx::warp_mbar_test_wait(done_bar(it + 1), done_parity(it + 1));
                 ptx::tmem_ld_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();

@@ -165,6 +165,17 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, v
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
     return mbar_wait_limit(bar, parity, abort_flag, WAIT_LIMIT_NS);
 }
+// The same for a whole warp, converged, ahead of warp-collective instructions (tcgen05.ld, tcgen05.st): the lanes leave together and
+// with one outcome, also when the phase completes between their probes or the wait runs out for some of them.
+__device__ __forceinline__ bool warp_mbar_wait(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag));
+}
+__device__ __forceinline__ bool warp_mbar_wait_hot(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait_hot(bar, parity, abort_flag));
+}
+__device__ __forceinline__ bool warp_mbar_test_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xFFFFFFFFu, mbar_test_wait(bar, parity));
+}
 
 // ---- flags in global memory between CTAs of one grid -------------------------------------------
 // sets the bits of v in *p; what this warp wrote before (and a __syncwarp ordered) is visible to who acquires them

@@ -30,6 +30,18 @@ def test_no_barrier_inside_the_roles_of_the_tensor_core_kernels():
         assert "named_bar_sync" not in text and "bar.sync" not in text and text.count("__syncthreads()") == 2, name
 
 
+def test_drain_warps_agree_ahead_of_tensor_memory_loads():
+    """tcgen05.ld is executed by whole warps: lanes that saw different outcomes of a look at a barrier, or of a wait that runs
+    out, must not part ways there.  The tall-tile kernel looks ahead, so each of its drain's looks and waits is the voting form."""
+    text = code("gemm_tcgen05.cu")
+    drain = text[text.index("setmaxnreg.inc"):text.index("bulk_wait_group0")]
+    assert "ready" in drain and "tmem_ld_32x32" in drain
+    assert not re.findall(r"(?<!warp_)mbar_(?:test_|try_)?wait\w*\(", drain)
+    for form in ("warp_mbar_wait", "warp_mbar_wait_hot", "warp_mbar_test_wait"):
+        body = re.search(r"bool " + form + r"\([^)]*\) \{(.*?)\n\}", code("ptx_sm100.cuh"), re.S).group(1)
+        assert "__all_sync(0xFFFFFFFFu" in body, form
+
+
 def test_shared_tables_read_in_16_byte_pieces_are_aligned():
     """A float2 table is 8-byte aligned by its type; where the compiler places it today is no promise."""
     text = code("streaming.cu")
