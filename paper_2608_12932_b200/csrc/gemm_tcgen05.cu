@@ -170,6 +170,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     static_assert(!SPLIT || C::SB * C::B_BYTES >= (TILE_M / 4 + TC_MAX_SPLIT - 1) * TILE_N * 16, "the split-K exchange buffer lives in the activation ring");
     static_assert(!(SPLIT && PC), "the per-channel form is not split along K");
     static_assert(!BAL || (!SPLIT && !PC), "the balanced walk is for the plain persistent form");
+    // Arrivals of one lane, of unpack and drain warps: a branch, or predicated instructions.  Each is the quicker one on its side (B200:
+    // 128 rows, per channel 4096 -> 4096 at 1024 tokens 21.1 us with branches, 22.5 predicated, grouped 4096 -> 24576 at 256
+    // 43.2 and 45.2; 208 rows at 1024 129.2 and 126.3, per channel 4096 -> 6144 22.3 and 21.8).
+    constexpr bool BRANCH = TILE_M <= 128;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -420,8 +424,15 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                ptx::mbar_arrive_if(bar(A_FULL + sa_), lane == 0);
-                ptx::mbar_arrive_if(bar(RAW_EMPTY + sr), lane == 0);
+                if (BRANCH) {
+                    if (lane == 0) {
+                        ptx::mbar_arrive(bar(A_FULL + sa_));
+                        ptx::mbar_arrive(bar(RAW_EMPTY + sr));
+                    }
+                } else {
+                    ptx::mbar_arrive_if(bar(A_FULL + sa_), lane == 0);
+                    ptx::mbar_arrive_if(bar(RAW_EMPTY + sr), lane == 0);
+                }
             }
         }
     } else {
@@ -516,10 +527,12 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
             __syncwarp();
             uint16_t sw_bits = next_sw_bits;
             if (PC) {
-                // one drain per tile: the buffer holds the sum of D over all groups (|sum| < 2^31 for K < 2^13 * 128)
+                // One drain per tile: the buffer holds the sum of D over all groups (|sum| < 2^31 for K < 2^13 * 128).  The wait lasts
+                // for the whole tile, so it parks: polling, the probes of eight warps queue up in front of the unpack's shared-memory
+                // accesses (4096 -> 4096 at 1024 tokens 24.8 us with polling, 22.5 parked; 4096 -> 6144, 208 rows, 23.4 and 21.8).
                 const uint32_t buf = tcount & 1u;
                 const float sw = __half2float(__ushort_as_half(sw_bits));
-                if (!(ok = ptx::warp_mbar_wait_hot(bar(TILE_DONE + buf), (tcount >> 1) & 1, abort_flag))) break;
+                if (!(ok = ptx::warp_mbar_wait(bar(TILE_DONE + buf), (tcount >> 1) & 1, abort_flag))) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t taddr = lane_taddr + buf * TILE_M;
                 uint32_t v[C::NCH][32];
@@ -576,7 +589,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                 ptx::tmem_ld_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
-                ptx::mbar_arrive_if(bar(ACC_EMPTY + buf), lane == 0);
+                if (!BRANCH) ptx::mbar_arrive_if(bar(ACC_EMPTY + buf), lane == 0);
+                else if (lane == 0) ptx::mbar_arrive(bar(ACC_EMPTY + buf));
 #pragma unroll
                 for (int ch = 0; ch < C::NCH; ++ch) {
 #pragma unroll

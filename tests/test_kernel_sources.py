@@ -42,6 +42,11 @@ def test_drain_warps_agree_ahead_of_tensor_memory_loads():
         assert "__all_sync(0xFFFFFFFFu" in body, form
 
 
+def test_waits_for_a_whole_tile_park():
+    """The per-channel drain waits as long as a tile takes; polling for that time slows the unpack warps beside it."""
+    assert re.findall(r"(\w*wait\w*)\(bar\(TILE_DONE", code("gemm_tcgen05.cu")) == ["warp_mbar_wait"]
+
+
 def test_shared_tables_read_in_16_byte_pieces_are_aligned():
     """A float2 table is 8-byte aligned by its type; where the compiler places it today is no promise."""
     text = code("streaming.cu")
