@@ -42,6 +42,8 @@ def check_ptxas(report):
         m2 = re.search(r"gemm_tc(?:gen05|short)_kernelILi\d+ELb(\d)E", name) or re.search(r"gemm_strip_kernelILi\d+ELi\d+ELb(\d)E", name)
         if m2 and m2.group(1) == "1":
             limit = 1024                          # the debug instantiations (partials dump) may spill
+        elif "gemm_tcgen05" in name:
+            limit = 0                             # whose roles have few registers each: a spill sits in a loop
         if spill > limit and "gemm_" in name:
             problems.append(f"{name}: {spill} bytes of spill stores")
         if "gemm_tcgen05" in name or "gemm_tcshort" in name:      # 512 and 640 threads share the 64 K registers

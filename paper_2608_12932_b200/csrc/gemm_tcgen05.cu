@@ -52,7 +52,7 @@
 // correction from the per-(token, channel, group) drain to the per-weight unpack.
 //
 // Warp roles (512 threads, four warpgroups so that setmaxnreg can move registers to the drain:
-// 40 / 40 / 216 / 216 per thread for 208-row tiles, 40 / 96 / 160 / 160 for shorter ones):
+// 40 / 40 / 216 / 216 per thread for 208-row tiles, 48 / 96 / 160 / 160 for shorter ones):
 //   warp 0       producer of the activation tiles (2-D TMA loads)
 //   warps 1, 3   MMA issuers (even and odd pipeline steps; an elected lane issues); warp 1 owns TMEM allocation
 //   warp 2       producer of the packed blobs (1-D bulk copies)
@@ -263,7 +263,8 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     const int runs_max = SPLIT ? (RUNS + S - 1) / S : 0;
     auto run_lo = [&](int o) { return RUNS * o / S; };
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (TILE_M > 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");          // (with 40 the split and the per-channel form spill)
         if (warp == WARP_PRODUCER && lane == 0) {
             // ------------------------------------------------ producer: activation tiles ----
             ptx::pdl_wait();                                    // the activations are the previous kernel's output
