@@ -172,8 +172,10 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
     static_assert(!BAL || (!SPLIT && !PC), "the balanced walk is for the plain persistent form");
     // Arrivals of one lane, of unpack and drain warps: a branch, or predicated instructions.  Each is the quicker one on its side (B200:
     // 128 rows, per channel 4096 -> 4096 at 1024 tokens 21.1 us with branches, 22.5 predicated, grouped 4096 -> 24576 at 256
-    // 43.2 and 45.2; 208 rows at 1024 129.2 and 126.3, per channel 4096 -> 6144 22.3 and 21.8).
-    constexpr bool BRANCH = TILE_M <= 128;
+    // 43.2 and 45.2; 208 rows at 1024 129.2 and 126.3, per channel 4096 -> 6144 22.3 and 21.8).  With a residual the branch, and no
+    // look ahead at the next step's barrier: both cost there, in the balanced walk above all (12288 -> 4096 at 1024 and 4096 tokens
+    // 71.1 and 296.9 us with both, 69.5 and 289.5 without; 13824 -> 5120 at 1391 126.2 and 123.6).
+    constexpr bool BRANCH = TILE_M <= 128 || RES, LOOK_AHEAD = !RES;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
@@ -586,7 +588,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_qa, const __grid_co
                     else ptx::tmem_ld_32x32(taddr + ch * 32, v[ch]);
                 }
                 // the next step's barrier, looked at under the loads' latency (past the last step: a phase that never completes)
-                ready = ptx::warp_mbar_test_wait(done_bar(it + 1), done_parity(it + 1));
+                if (LOOK_AHEAD) ready = ptx::warp_mbar_test_wait(done_bar(it + 1), done_parity(it + 1));
                 ptx::tmem_ld_wait();
                 ptx::tc_fence_before_sync();
                 __syncwarp();
