@@ -75,9 +75,10 @@ size_t w4a8_packed_bytes(int N, int K, int group);
  * per-tile arrival counters and hand-over flags; the strip kernel's hand-over slots; one status
  * word); 0 for an unsupported shape.  The first W4A8_WORKSPACE_ZEROED_BYTES bytes (or the whole
  * workspace, if it is smaller) must be zero before the first call (w4a8_workspace_init does that)
- * and are left by every call as the next one needs them (zero, but for the fused gate+up call's
- * maxima, which carry the numbers of their calls), so one workspace can serve any number of calls that do not
- * overlap on the GPU.
+ * and are left by every call as the next one needs them, so one workspace can serve any number of calls that do not
+ * overlap on the GPU.  "As the next one needs them" is zero, but for bytes 64 to 207: the strip-kernel forms of
+ * w4a8_gate_up_silu_quantize keep their per-token maxima and call numbers there from call to call.  Zeroing all of
+ * the workspace between calls is always allowed; zeroing a part of those bytes is not.
  */
 #define W4A8_WORKSPACE_HEADER_BYTES 4096
 #define W4A8_WORKSPACE_ZEROED_BYTES (4096 + 192 * 16384)
@@ -212,8 +213,10 @@ w4a8_status w4a8_gemm_residual(w4a8_path path, const int8_t* qa, const uint16_t*
  *              warps that quantise it (required)
  *   y_scratch  device, bf16 [M, N]; needed only by the SEPARATE form, else may be NULL
  * Errors as for w4a8_gemm; W4A8_ERR_SHAPE also for I % 128 != 0, an unknown form, or a strip-kernel form where that kernel
- * does not exist (M > 16).  The strip-kernel forms keep 18 words of the workspace header (per-token maxima and two
- * counters) that they leave zero; after W4A8_ERR_TIMEOUT the workspace must be initialised again before its next use.
+ * does not exist (M > 16).  The strip-kernel forms keep 38 words of the workspace header, bytes 64 to 215: sixteen 64-bit
+ * per-token maxima, each with the number of its call above 16 bits of magnitude, and two 64-bit call numbers, none of which is ever
+ * cleared, then two 32-bit counters that every call leaves zero.  After W4A8_ERR_TIMEOUT the workspace must be initialised
+ * again before its next use.
  */
 typedef enum {
     W4A8_GATE_UP_AUTO = 0,

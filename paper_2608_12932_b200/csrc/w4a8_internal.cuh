@@ -39,12 +39,13 @@ constexpr int BLOB_BYTES = BLOB_ZERO_OFF + TILE_N / 2;        // 8512
 
 // ---- workspace layout -----------------------------------------------------------------------
 //   [0, 4)                    status word (0 = fine, else a w4a8_status written by a kernel)
+//   [64, 216)                 fused gate+up form (FuseSync below): maxima and call numbers stay, the counters are zero between calls
 //   [256, 256 + 4*n_tiles)    split-K arrival counters, one per 128-channel tile (zero between calls)
 //   [HEADER, SHARED)          hand-over slots of the strip kernel: one per CTA, each word a float and a tag
 //                             (all zero between calls: the tag is what says that a word has been written)
 //   [SHARED, ...)             split-K fp32 slices  [S][M][N], or the tensor-core kernel's hand-over tiles
 constexpr int WS_STATUS_OFF = 0;
-constexpr int WS_FUSE_SYNC_OFF = 64;    // fused gate+up form (FuseSync): maxima, call counts, arrivals, departures
+constexpr int WS_FUSE_SYNC_OFF = 64;
 // Each maximum carries the number of its call above 16 bits of magnitude, so a call's first maximum supersedes whatever an earlier
 // call left: nothing has to be cleared, and no kernel has to learn that every reader is done.  The projection takes the number
 // from `done` (calls that are complete) and leaves it in `running`; the kernel that quantises h takes it from there and, at any time,
@@ -54,7 +55,7 @@ struct FuseSync {
     unsigned long long done, running;
     uint32_t arrivals, departures;      // one-kernel form; zero between calls
 };
-static_assert(WS_FUSE_SYNC_OFF % 8 == 0 && WS_FUSE_SYNC_OFF + sizeof(FuseSync) <= 256, "in front of the counters");
+static_assert(WS_FUSE_SYNC_OFF == 64 && sizeof(FuseSync) == 152, "bytes 64 to 215, as the public header says; in front of the split-K counters");
 constexpr int WS_COUNTER_OFF = 256;
 constexpr int WS_HEADER_BYTES = W4A8_WORKSPACE_HEADER_BYTES;
 constexpr int MAX_N_TILES = (WS_HEADER_BYTES - WS_COUNTER_OFF) / 4;   // 960 tiles = N up to 122880

@@ -43,3 +43,37 @@ def test_a_used_workspace_gives_the_bits_of_a_fresh_one(M):
             qa, sa, asum = onp.quantize_act(bits(got[0]), 128)
             assert np.array_equal(got[1].cpu().numpy(), qa) and np.array_equal(bits(got[2]), sa) and np.array_equal(got[3].cpu().numpy(), asum)
             assert bits(got[2])[M // 2] == 0
+
+
+def layers(I, K):
+    gu, down = wl.make_layer(K, 2 * I, 11, 4), wl.make_layer(I, K, 12, 4)
+    return [B.w4a8_pack_weights(torch.from_numpy(c["qw"]).cuda(), t_u16(c["sw"], torch.float16), torch.from_numpy(c["z"]).cuda()) for c in (gu, down)]
+
+
+def workspace(I, K):
+    return max((B.new_workspace(16, *nk) for nk in ((2 * I, K), (K, I))), key=lambda w: w.numel())
+
+
+def step(x, gu, down, I, K, ws, form, other):
+    """One fused step and the down projection behind it; `other`: a call of another kernel family on the workspace between them."""
+    q = B.w4a8_quantize_act(x)
+    out = B.w4a8_gate_up_silu_quantize(*q, gu, 2 * I, ws, form=form)
+    if other:
+        B.w4a8_gemm(*q, gu, 2 * I, ws, path=other)
+    return [*out, B.w4a8_gemm(*out[1:], down, K, ws)]
+
+
+@pytest.mark.parametrize("form", [B.GATE_UP_EPILOGUE, B.GATE_UP_ONE_KERNEL])
+def test_what_a_call_leaves_in_the_workspace(form):
+    """As the public header says it: bytes 64 to 207 hold maxima and call numbers, all else of the zeroed part is zero again."""
+    I, K = 6144, 1280
+    gu, down = layers(I, K)
+    ws = workspace(I, K)
+    rng = np.random.default_rng(3)
+    for M in (16, 5, 8):
+        step(t_u16(bf16_bits(rng.standard_normal((M, K))), torch.bfloat16), gu, down, I, K, ws, form, None)
+    B.w4a8_check_status(ws)
+    left = ws[:4096 + 192 * 16384].cpu().numpy()
+    words = left[64:208].view(np.uint64)
+    assert (words[:16] >> np.uint64(16)).max() == 3 and (words[:16] & np.uint64(0xFFFF)).all() and words[16] == 3
+    assert not left[:64].any() and not left[208:].any()

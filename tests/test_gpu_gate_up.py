@@ -117,7 +117,7 @@ def test_gate_up_forms_against_oracle_and_one_another(M, K, I):
     groups = {}
     for form in forms:
         in_strip = form in (B.GATE_UP_EPILOGUE, B.GATE_UP_ONE_KERNEL) or strip
-        for rep in range(3):                                   # the workspace words must come back to zero each time
+        for rep in range(3):                                   # each call must leave the workspace ready for the next
             h, qa_h, sa_h, asum_h = B.w4a8_gate_up_silu_quantize(qa, sa, asum, packed, N, ws, form=form)
             torch.cuda.synchronize()
             B.w4a8_check_status(ws)
