@@ -126,9 +126,9 @@ w4a8_status w4a8_quantize_act(const void* x_bf16, int M, int K, int group,
  * Programmatic dependent launch: w4a8_quantize_act, the weight-streaming kernels for up to 64
  * tokens and the tensor-core kernel are launched with programmatic stream serialisation (only the
  * workspace variant of the split-K kernel is launched plainly).  When consecutive library calls share a
- * stream, such a kernel may start, and prefetch packed weights, before its predecessor in the
- * stream has finished; it waits on the device before it reads any activation, token scale or group
- * sum, touches the workspace or writes any output.  packed_w is therefore the one argument that
+ * stream, such a kernel may start, read packed weights and ask for x_bf16 to be brought into the L2 cache (which
+ * reads no value of it) before its predecessor in the stream has finished; it waits on the device before it
+ * reads any activation, token scale or group sum, touches the workspace or writes any output.  packed_w is therefore the one argument that
  * must be complete before the call is enqueued: do not produce it with a kernel that sits
  * immediately ahead of the GEMM in the same stream (weights are packed once, offline).
  */

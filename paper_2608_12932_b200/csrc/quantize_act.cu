@@ -78,13 +78,16 @@ __global__ void __launch_bounds__(QA_THREADS, QA_THREADS == 256 ? (QA_CACHE == 2
 quantize_act_kernel(const uint4* __restrict__ x, int K, uint2* __restrict__ qa,
                     uint16_t* __restrict__ sa, int32_t* __restrict__ asum, uint4* __restrict__ h_out) {
     // Under programmatic dependent launch this grid may start while its predecessor still runs:
-    // let the next grid start as early, and touch no memory before the predecessor is complete.
+    // let the next grid start as early, and read and write nothing before the predecessor is complete.
     ptx::pdl_launch_dependents();
     if (!SILU && !COPY && QA_THREADS >= 512) {
-        // Few rows: the row is asked into L2 ahead of the wait, a line per thread and turn; behind the wait it would queue with the
-        // weights that the next kernel already requests.  (Decoder layers of 4096 and 5120 channels at 2 to 16 tokens, where two of the
-        // quantised inputs are cold: 39.3 and 37.9 us at 2 and 8 tokens, now 38.3 and 37.6; 49.1 at 8 of the larger, 47.7.  Not where x may
-        // lie in host memory, which is the COPY form.)
+        // Up to 512 rows: the row is asked into L2 ahead of the wait, a line per thread and turn; behind the wait it would queue with the
+        // weights that the next kernel already requests.  What the predecessor still has to write is written in L2, so a line asked
+        // for too early is not stale.  Measured on B200 over 1 to 512 rows, without the request and with it.  x cold: 4096 -> 6144 as
+        // w4a8_linear 6.5 and 6.2 us at 1 and 8 rows, 8.9 and 8.7 at 17, 11.7 and 11.5 at 64, equal at 128, 20.4 and 20.2 at 300; the quantiser alone
+        // 2.5 and 2.1 at 64, 2.9 and 2.6 at 200, 4.7 and 4.4 at 512, up to 16 rows 0.06 us the other way.  x written by the kernel before:
+        // w4a8_linear within 1 % at most counts, 9.7 and 9.9 at 8, 11.9 and 11.9 at 16, 12.7 and 12.8 at 17, 28.3 and 28.3 at 512.  Not with
+        // more rows, where it was not measured, nor where x may lie in host memory, which is the COPY form.
         const uint4* row = x + (size_t)blockIdx.x * (K >> 3);
         for (int c = threadIdx.x * 8; c < (K >> 3); c += QA_THREADS * 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + c));
     }
