@@ -77,3 +77,51 @@ def test_what_a_call_leaves_in_the_workspace(form):
     words = left[64:208].view(np.uint64)
     assert (words[:16] >> np.uint64(16)).max() == 3 and (words[:16] & np.uint64(0xFFFF)).all() and words[16] == 3
     assert not left[:64].any() and not left[208:].any()
+
+
+def same(got, want):
+    return all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got, want, strict=True))
+
+
+# 1280 -> 2 x 6144: 384 strips of 32 channels in two stages each, more than there are CTAs, so that neighbours share strips
+@pytest.mark.parametrize("M,I,K", [(1, 256, 256), (8, 256, 256), (16, 2432, 1024), (1, 6144, 1280), (8, 6144, 1280), (16, 6144, 1280)])
+def test_steps_behind_one_another(M, I, K):
+    """Nothing waits on the host between the calls, so a call's kernels start while the last call's still run: large and small
+    values, both token counts, both forms and other kernel families in turn, then the same captured and replayed."""
+    plan = B.w4a8_plan(M, 2 * I, K)
+    if I == 6144 and M <= 8:
+        assert plan["strip_rows"] == 32 and any(768 * c // plan["ctas"] % 2 for c in range(plan["ctas"]))
+    gu, down = layers(I, K)
+    rng = np.random.default_rng(M + I)
+    bf = lambda m, scale: t_u16(bf16_bits(rng.standard_normal((m, K)) * scale), torch.bfloat16)
+    seq = [(bf(16, 100.0), B.GATE_UP_EPILOGUE, None), (bf(M, 0.01), B.GATE_UP_EPILOGUE, None), (bf(M, 1.0), B.GATE_UP_ONE_KERNEL, None),
+           (bf(M, 0.01), B.GATE_UP_EPILOGUE, B.PATH_SPLITK), (bf(16, 10.0), B.GATE_UP_ONE_KERNEL, B.PATH_TCGEN05),
+           (bf(M, 0.1), B.GATE_UP_ONE_KERNEL, None), (bf(M, 0.01), B.GATE_UP_EPILOGUE, B.PATH_TCGEN05), (bf(M, 0.02), B.GATE_UP_EPILOGUE, None)]
+    if M > 1:
+        for x, _, _ in seq[1:]:
+            x[x.shape[0] // 2] = 0                             # a token whose h is zero throughout leaves its old maximum in place
+    want = []
+    for x, form, other in seq:
+        ws = workspace(I, K)
+        want.append(step(x, gu, down, I, K, ws, form, other))
+        B.w4a8_check_status(ws)
+    assert all(bits(w[2]).any() for w in want)                 # scales of h that are not zero: maxima were written
+    used = workspace(I, K)
+    torch.cuda.synchronize()
+    got = [step(x, gu, down, I, K, used, form, other) for _ in range(3) for x, form, other in seq]
+    B.w4a8_check_status(used)
+    assert all(same(g, want[i % len(seq)]) for i, g in enumerate(got))
+
+    x = seq[1][0].clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = [step(x, gu, down, I, K, used, form, None) for form in (B.GATE_UP_EPILOGUE, B.GATE_UP_ONE_KERNEL, B.GATE_UP_EPILOGUE)]
+    pick = [k for k in range(len(seq)) if seq[k][0].shape[0] == M]
+    kept = []
+    for k in pick * 2:
+        x.copy_(seq[k][0])
+        graph.replay()
+        kept.append((k, [[t.clone() for t in o] for o in out]))
+    B.w4a8_check_status(used)
+    for k, outs in kept:
+        assert all(same(o, want[k]) for o in outs), k
