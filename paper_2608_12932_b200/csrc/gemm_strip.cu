@@ -99,7 +99,7 @@ __host__ __device__ inline StLayout st_layout(int mb, int rblk, int stages, int 
     L.take_off = L.part_off + ST_CONSUMER_WARPS * (rblk >= 2 ? 2 : 1) * mb * 32 * 16;   // one float4 per consumer lane, row block and token block
     L.ystage_off = L.take_off + rblk * mb * 32 * 16;        // the neighbour's sums of a shared strip
     // a strip's outputs, [token][channel], rows padded by 16 B: bf16, or fp32 when a residual is added at the store
-    L.misc_off = L.ystage_off + mp * ((fp32_stage ? 64 : 32) * rblk + 16);
+    L.misc_off = L.ystage_off + mp * ((fp32_stage ? 64 : 32) * rblk + 16);     // abort flag; one-kernel fused form: place, call number
     L.total = L.misc_off + 16;
     return L;
 }
@@ -712,6 +712,7 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
                 uint32_t place;
                 asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(place) : "l"(&a.sync->arrivals) : "memory");
                 *reinterpret_cast<volatile uint32_t*>(smem + L.misc_off + 4) = place;
+                *reinterpret_cast<volatile unsigned long long*>(smem + L.misc_off + 8) = call;
             }
         }
         if (lane == 0) ST_STAMP(6);
@@ -727,6 +728,10 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
         const uint32_t place = *reinterpret_cast<volatile uint32_t*>(smem + L.misc_off + 4);
         if (tid == 0) { ST_STAMP(7); ST_PUT(12, place); }
         if (place >= gridDim.x - stay) {
+            // The call's number comes out of shared memory, where the epilogue warp left it: read again from `done` by every stayer,
+            // and once more by the last to leave, it was two round trips to L2 in the tail of the launch (2048 -> 2 x 6144 at 8
+            // tokens 10.4 us, now 9.2; 4096 -> 2 x 12288 17.4, now 15.8).
+            const unsigned long long call = *reinterpret_cast<volatile unsigned long long*>(smem + L.misc_off + 8);
             const uint32_t rank = place - (gridDim.x - stay);
             if (tid == 0) {
                 uint64_t t0 = 0;
@@ -747,7 +752,6 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
             if (!*abort_flag) {
                 const int I = a.N / 2, Gh = I / GROUP;
                 constexpr int WARPS = ST_THREADS / 32;
-                const unsigned long long call = __ldcg(&a.sync->done) + 1;      // the last stayer to leave moves it on
                 for (int u = (int)rank * WARPS + warp; u < a.M * Gh; u += (int)stay * WARPS)
                     requant_unit(a.h, I, Gh, u, lane, a.qa_h, a.sa_h, a.asum_h, a.sync, call);
             }
@@ -757,7 +761,7 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
             if (tid == 0) {
                 const uint32_t old = atomicAdd(&a.sync->departures, 1u);
                 if (old == stay - 1) {
-                    a.sync->done += 1;
+                    a.sync->done = call;
                     a.sync->arrivals = a.sync->departures = 0u;
                     __threadfence();
                 }

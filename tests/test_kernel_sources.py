@@ -47,6 +47,14 @@ def test_waits_for_a_whole_tile_park():
     assert re.findall(r"(\w*wait\w*)\(bar\(TILE_DONE", code("gemm_tcgen05.cu")) == ["warp_mbar_wait"]
 
 
+def test_a_calls_number_is_read_once():
+    """In the fused gate+up step's one-kernel form every further read of the number would be a round trip in the launch's tail."""
+    text = code("gemm_strip.cu")
+    text = text[text.index("gemm_strip_kernel("):text.index("requant_kernel(")]
+    assert text.count("__ldcg(&a.sync->done)") == 1
+    assert re.findall(r"sync->done ([^;]*);", text) == ["= call"]
+
+
 def test_shared_tables_read_in_16_byte_pieces_are_aligned():
     """A float2 table is 8-byte aligned by its type; where the compiler places it today is no promise."""
     text = code("streaming.cu")
