@@ -345,7 +345,7 @@ def run_large_m_roofline(torch, B, peaks, l2_bytes, timer):
            "peak_source": f"2 x the {peaks['source']} bf16 GEMM rate (burst); nominal dense int8 : bf16 = 2",
            "frac": round(tops / peak2, 4), "us_per_launch": round(us, 2),
            "frac_of_nominal_4500": round(tops / NOMINAL_INT8_TOPS, 4),
-           "tensor_pipe_active_pct_ncu": 33.5, "traffic": None,
+           "tensor_pipe_active_pct_ncu": 35.4, "traffic": None,
            "timing": "median of 5 replays of back-to-back launches in one graph"}
     if peaks.get("int8_tops_burst"):
         out["peak_int8_mm"] = round(peaks["int8_tops_burst"], 1)
@@ -839,7 +839,7 @@ def run_rope(args):
 # dram__bytes_read.sum + dram__bytes_write.sum of one GEMM launch at the headline shape, by kernel, from the ncu
 # captures summarised under profiles/ (gemm_strip_qkv_M8.md, gemm_cluster_qkv_M8.md)
 QUANTIZE_TRAFFIC_BYTES_PER_LAUNCH = 8410624      # ncu, quantize_act at 1024 x 4096 (profiles/quantize_act_M1024_K4096.md)
-TRAFFIC_BYTES_PER_LAUNCH = {"gemm_strip_kernel": 13148416, "gemm_cluster_kernel": 13144832}
+TRAFFIC_BYTES_PER_LAUNCH = {"gemm_strip_kernel": 13142528, "gemm_cluster_kernel": 13144832}
 E2E_DEPTH = int(os.environ.get("W4A8_E2E_DEPTH", "8"))          # host requests in flight in the end-to-end measurement
 
 

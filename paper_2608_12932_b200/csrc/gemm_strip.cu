@@ -245,8 +245,9 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
     const StLayout L = st_layout(MB, RBLK, stages, G, FUSE == 3);
     // The warp index comes out of a shuffle, so that the compiler knows it to be warp-uniform: the roles' loop counters, ring and
     // barrier addresses then live on the uniform datapath.  (B200, one launch behind another, cold weights, before and after:
-    // 4096 -> 24576 at 1, 8 and 16 tokens 13.8, 13.7 and 17.8 us, 13.3, 13.1 and 16.8; 4096 -> 6144 at 8 5.1, 4.8; 12288 -> 4096 with
-    // residual at 8 and 16 7.9 and 10.3, 7.5 and 9.6; warp instructions of the first at 8 tokens 5.69 M, 5.37 M.)
+    // 4096 -> 24576 at 1, 8 and 16 tokens 11.8, 11.7 and 14.5 us, 11.6, 11.4 and 13.7; 4096 -> 6144 at 8 5.1, 4.8; 12288 -> 4096 with
+    // residual at 8 and 16 7.5 and 9.5, 7.2 and 8.9; warp instructions of the first at 8 tokens 5.69 M, 5.37 M, and 5.19 M since the requests for the rest of
+    // the layer into L2 went.)
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
 
     // this CTA's contiguous range of stages, [lo, hi), and the strips it touches
@@ -304,7 +305,8 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tm_act, const __grid_const
         // (What the ring cannot hold is not asked into L2 meanwhile: requests for a whole layer at once delay the kernel that this one
         // waits for - the quantiser, or the last stores of the projection before - by more than they bring.  4096 -> 24576 at 1, 8 and
         // 16 tokens behind one another 13.2, 13.2 and 16.7 us with such requests, 11.5, 11.4 and 13.8 without; 12288 -> 4096 with
-        // residual at 16 9.5 and 8.7; behind the quantiser the same layer 15.7 and 13.7 at 8 tokens, 12288 -> 4096 10.1 and 10.4.)
+        // residual at 16 9.5 and 8.7; behind the quantiser the same layer 15.7 and 13.7 at 8 tokens.  12288 -> 4096 behind the quantiser at
+        // 8 tokens is the one size that gains nothing: 10.9 and 10.8 in a chain, 17.2 and 17.3 alone with a cold L2.)
     }
     // Activations, their scales and group sums, and the workspace belong to the previous kernel until
     // this wait returns.  They are read only after it and only through L2 (TMA, ld.global.cg).

@@ -17,8 +17,8 @@
 // its columns are in registers.
 //
 // The tensor pipe is not what bounds this kernel (it is busy under a third of the time): the CUDA
-// cores must take every accumulator element out of TMEM after every group and spend two
-// instructions on it, the unpack shares the integer pipe with that conversion, and shared memory
+// cores must take every accumulator element out of TMEM after every group and spend one and
+// a half instructions on it, the unpack shares the integer pipe with that conversion, and shared memory
 // (about 128 B/clk per SM) is shared by the tensor core's operand reads, the bulk-copy fills and
 // ordinary loads.  Design choices made on measurements:
 //  * the unpacked weights never touch shared memory: an unpack thread owns one weight row
@@ -38,10 +38,12 @@
 //  * what paces a step of a 208-row tile is the chain of a drain warp - the look at its barrier, the loads, the hand-back and the
 //    sums, 100 to 200 cycles for each of the first three however long ago the MMAs finished (measured with stamps; the
 //    barrier has completed at the first look five times out of six).  So the warp index is made warp-uniform (ring indices,
-//    barrier and tensor-memory addresses on the uniform datapath), arrivals are predicated instructions instead of one-lane
-//    branches, the next step's barrier is looked at under the loads, and two sums take one packed FMA: 4096 -> 24576 at 1024
-//    and 4096 tokens 132.4 and 523 us before, 125.4 and 491 after, 4096 -> 6144 40.2 and 132, 38.3 and 125.7; with a residual
-//    0 to 4 % (B200, weights cold).  Tried on top, none quicker: the conversion moved to the FMA pipe by a constant bias in the
+//    barrier and tensor-memory addresses on the uniform datapath) and two sums take one packed FMA; in 208-row tiles without a
+//    residual arrivals are predicated instructions instead of one-lane branches, and without a residual, at every height, the
+//    next step's barrier is looked at under the loads (where these two cost instead, they are not taken: see BRANCH below).
+//    Together, 4096 -> 24576 at 1024 and 4096 tokens 132.2 and 521 us before, 127.2 and 471 after, 4096 -> 6144 43.8 and 138.3, 41.7
+//    and 131.9, 5120 -> 27648 at 1391 241.5 and 237.0; with a residual 12288 -> 4096 at 1024 and 4096 70.5 and 273.9, 69.6 and 269.9,
+//    4096 -> 4096 equal (B200, weights cold, both builds in turn).  Tried on top, none quicker: the conversion moved to the FMA pipe by a constant bias in the
 //    accumulators (131), for half of the columns (134), the two halves of the columns filled and handed back on their own (144),
 //    columns loaded in pieces ahead of the sums (129.6), a tile's outputs staged whole (127.4 before the look ahead, equal);
 //  * one tcgen05.commit per step, on a ring of "step done" barriers, frees the step's weight and
